@@ -10,10 +10,10 @@
 //
 // All contractions run on the 5th-generation tensor cores (tcgen05.mma,
 // kind::f16, BF16 operands from shared memory, FP32 accumulator in tensor
-// memory).  One GEMM kernel serves every layer:
-//   forward  Z_l  = H_{l-1} W_l^T          A = H [rows][in],  B = W  [out][in]
-//   backward dH   = dZ_l W_l               A = dZ [rows][out], B = W^T [in][out]
-//   gradient dW_l = dZ_l^T H_{l-1}         A = dZ^T [out][rows], B = H^T [in][rows] (split over rows)
+// memory).  Inference and the forward pass of training run one fused kernel
+// (k_mlp_infer_pair); the backward pass and the weight gradients are in
+// ens_train.cuh.  A plain GEMM kernel per layer (k_gemm_tc) remains as the
+// layer-by-layer forward pass that checks the fused one.
 #include "../../include/ens.h"
 #include "ens_internal.h"
 #include "ens_tc.cuh"
@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace ens {
@@ -200,8 +201,7 @@ __device__ void row_features(const RowSpec &rs, double lam, int bin, float *f)
     }
 }
 
-__global__ void k_features(RowSpec rs, const double *lams, int nlam, long long rows_pad, __nv_bfloat16 *X,
-                           __nv_bfloat16 *Xt)
+__global__ void k_features(RowSpec rs, const double *lams, int nlam, long long rows_pad, __nv_bfloat16 *X)
 {
     const long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= rows_pad) return;
@@ -212,13 +212,10 @@ __global__ void k_features(RowSpec rs, const double *lams, int nlam, long long r
     } else {
         for (int i = 0; i < kIn; ++i) f[i] = 0.f;
     }
-    for (int i = 0; i < kIn; ++i) {
-        X[row * kIn + i] = __float2bfloat16(f[i]);
-        if (Xt) Xt[(long long)i * rows_pad + row] = __float2bfloat16(f[i]);
-    }
+    for (int i = 0; i < kIn; ++i) X[row * kIn + i] = __float2bfloat16(f[i]);
 }
 
-// sigmoid(z) = (1 + tanh(z/2)) / 2 with the hardware tanh approximation: one
+// sigmoid(z) = (1 + tanh(z/2)) / 2 from the hardware tanh approximation: one
 // special-function-unit operation per element (the epilogues are bound by
 // that unit), relative error far below the BF16 rounding of the activations
 __device__ __forceinline__ float tanh_approx(float x)
@@ -227,18 +224,11 @@ __device__ __forceinline__ float tanh_approx(float x)
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float sigmoid(float z) { return fmaf(0.5f, tanh_approx(0.5f * z), 0.5f); }
 // SiLU z sigmoid(z) written with h = z / 2 as h + h tanh(h): two FMAs and one
 // tanh (the fused inference forms h = v / 2 + b / 2 in one FMA with halved
 // biases, bit for bit the same h as (v + b) / 2)
 __device__ __forceinline__ float silu_h(float h) { return fmaf(h, tanh_approx(h), h); }
 __device__ __forceinline__ float silu(float z) { return silu_h(0.5f * z); }
-__device__ __forceinline__ float dsilu(float z)
-{
-    const float s = sigmoid(z);
-    return s * (1.f + z * (1.f - s));
-}
-
 // BF16 rounding (round to nearest, ties to even) on the integer pipe: the
 // upper 16 bits of the result are the BF16 of f, bit for bit the conversion
 // instruction's result for every non-NaN f (a NaN stays a NaN).
@@ -261,9 +251,6 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi)
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// f rounded to BF16, as FP32
-__device__ __forceinline__ float round_bf16(float f) { return __uint_as_float(bf16_rne_bits(f) & 0xFFFF0000u); }
-
 // a * b + c on both halves with one packed FP32x2 instruction (each half
 // rounded as the scalar FMA)
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
@@ -283,18 +270,12 @@ __device__ __forceinline__ float2 silu_pair(float2 v, float2 bh)
     return fma2(h, make_float2(tanh_approx(h.x), tanh_approx(h.y)), h);
 }
 
-// Z += bias (kept, FP32, for the backward pass); H = SiLU(Z) as BF16 (and H^T)
-__global__ void k_bias_silu(float *Z, const float *bias, long long rows, __nv_bfloat16 *H, __nv_bfloat16 *Ht)
+// H = SiLU(Z + bias) as BF16 (layer-by-layer forward pass)
+__global__ void k_bias_silu(const float *Z, const float *bias, long long rows, __nv_bfloat16 *H)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * kHid) return;
-    const long long row = i / kHid;
-    const int c = (int)(i % kHid);
-    const float z = Z[i] + bias[c];
-    Z[i] = z;
-    const __nv_bfloat16 h = __float2bfloat16(silu(z));
-    H[i] = h;
-    if (Ht) Ht[(long long)c * rows + row] = h;
+    H[i] = __float2bfloat16(silu(Z[i] + bias[i % kHid]));
 }
 
 // logit = H3 . w4 + b4, one warp per row
@@ -372,68 +353,6 @@ __global__ void k_softmax_ce(const float *logit, const float *target, int nq, in
     }
 }
 
-// dZ3 = (dlogit w4^T) * SiLU'(Z3) as BF16 (and dZ3^T); rows beyond `real` are zero
-__global__ void k_head_back(const float *dlogit, const float *w4, const float *Z, long long rows, long long real,
-                            __nv_bfloat16 *dZ, __nv_bfloat16 *dZt)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * kHid) return;
-    const long long row = i / kHid;
-    const int c = (int)(i % kHid);
-    const float v = row < real ? dlogit[row] * w4[c] * dsilu(Z[i]) : 0.f;
-    const __nv_bfloat16 b = __float2bfloat16(v);
-    dZ[i] = b;
-    dZt[(long long)c * rows + row] = b;
-}
-
-// dZ = dH * SiLU'(Z) as BF16 (and dZ^T)
-__global__ void k_silu_back(const float *dH, const float *Z, long long rows, __nv_bfloat16 *dZ, __nv_bfloat16 *dZt)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * kHid) return;
-    const long long row = i / kHid;
-    const int c = (int)(i % kHid);
-    const __nv_bfloat16 b = __float2bfloat16(dH[i] * dsilu(Z[i]));
-    dZ[i] = b;
-    dZt[(long long)c * rows + row] = b;
-}
-
-// column sums over rows of a BF16 [rows][kHid] matrix (bias gradients) and
-// of dlogit * H (head weight gradient), deterministic: one block per column
-__global__ void k_colsum_bf16(const __nv_bfloat16 *M, long long rows, float *out)
-{
-    const int c = blockIdx.x;
-    float s = 0.f;
-    for (long long r = threadIdx.x; r < rows; r += blockDim.x) s += __bfloat162float(M[r * kHid + c]);
-    __shared__ float red[32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        out[c] = t;
-    }
-}
-
-__global__ void k_head_grad(const float *dlogit, const __nv_bfloat16 *H, long long real, float *gw4, float *gb4)
-{
-    const int c = blockIdx.x;   // 0..kHid (kHid: bias)
-    float s = 0.f;
-    for (long long r = threadIdx.x; r < real; r += blockDim.x)
-        s += dlogit[r] * (c < kHid ? __bfloat162float(H[r * kHid + c]) : 1.f);
-    __shared__ float red[32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        if (c < kHid) gw4[c] = t;
-        else gb4[0] = t;
-    }
-}
-
 // sum of split-K partials (fixed order)
 __global__ void k_sum_splits(const float *part, int splits, long long n, float *out)
 {
@@ -485,10 +404,19 @@ __device__ __forceinline__ uint32_t wimg_offset(int o, int k)
     return (uint32_t)((k >> 6) * 32768) + sw128_offset(o, k & 63);
 }
 
-// BF16 operand copies: W1 [256][64], W2/W3 [256][256] and their transposes,
-// and (optional) the swizzled shared-memory images of W1, W2, W3 that the
-// fused inference kernel copies in with bulk copies
-__global__ void k_pack_weights_img(const float *p, unsigned char *img1, unsigned char *img2, unsigned char *img3)
+// biases and head weights of the fused kernels: read by value from the
+// constant bank (inference: warp-uniform addresses, broadcasts) or from
+// memory (training, where they change every step without a host round trip)
+struct MlpBias {
+    float b1[kHid], b2[kHid], b3[kHid];   // halved: the epilogues form (z + b) / 2 in one FMA (exact in FP32)
+    float w4[kHid];
+    float b4;
+};
+
+// Operands of the fused kernels from the FP32 parameters: the swizzled BF16
+// shared-memory images of W1, W2, W3 (bulk copies) and the biases and head
+__global__ void k_pack_weights_img(const float *p, unsigned char *img1, unsigned char *img2, unsigned char *img3,
+                                   MlpBias *bias)
 {
     const ParamLayout L = param_layout();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -501,21 +429,24 @@ __global__ void k_pack_weights_img(const float *p, unsigned char *img1, unsigned
         *reinterpret_cast<__nv_bfloat16 *>(img2 + wimg_offset(o, k)) = __float2bfloat16(p[L.W2 + i]);
         *reinterpret_cast<__nv_bfloat16 *>(img3 + wimg_offset(o, k)) = __float2bfloat16(p[L.W3 + i]);
     }
+    if (i < kHid) {
+        bias->b1[i] = 0.5f * p[L.b1 + i];
+        bias->b2[i] = 0.5f * p[L.b2 + i];
+        bias->b3[i] = 0.5f * p[L.b3 + i];
+        bias->w4[i] = p[L.w4 + i];
+    }
+    if (i == 0) bias->b4 = p[L.b4];
 }
 
-__global__ void k_pack_weights(const float *p, __nv_bfloat16 *W1b, __nv_bfloat16 *W2b, __nv_bfloat16 *W3b,
-                               __nv_bfloat16 *W2t, __nv_bfloat16 *W3t)
+// BF16 weights W1 [256][64], W2, W3 [256][256] of the layer-by-layer forward pass
+__global__ void k_pack_weights(const float *p, __nv_bfloat16 *W1b, __nv_bfloat16 *W2b, __nv_bfloat16 *W3b)
 {
     const ParamLayout L = param_layout();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < (long long)kHid * kIn) W1b[i] = __float2bfloat16(p[L.W1 + i]);
     if (i < (long long)kHid * kHid) {
-        const int o = (int)(i / kHid), c = (int)(i % kHid);
-        const __nv_bfloat16 w2 = __float2bfloat16(p[L.W2 + i]), w3 = __float2bfloat16(p[L.W3 + i]);
-        W2b[i] = w2;
-        W3b[i] = w3;
-        W2t[(long long)c * kHid + o] = w2;
-        W3t[(long long)c * kHid + o] = w3;
+        W2b[i] = __float2bfloat16(p[L.W2 + i]);
+        W3b[i] = __float2bfloat16(p[L.W3 + i]);
     }
 }
 
@@ -593,13 +524,56 @@ __global__ void k_feature_table(RowSpec rs, const double *lams, int nlam, uint4 
     for (int j = 0; j < kIn / 8; ++j) ftab[(long long)i * (kIn / 8) + j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
 }
 
-// biases and head weights by value: kernel parameters live in the constant
-// bank, read in pairs by the epilogues (warp-uniform addresses: broadcasts)
-struct MlpBias {
-    float b1[kHid], b2[kHid], b3[kHid];   // halved: the epilogues form (z + b) / 2 in one FMA
-    float w4[kHid];
-    float b4;
+// 16 per-column parameters of an epilogue chunk as pairs, from memory by four
+// 16-byte loads placed where they are written: hoisted by the compiler, or
+// fetched a chunk ahead, they spill (96 registers per thread; the backward
+// kernel took 344 us against 296)
+struct Cols16 {
+    float2 v[8];
+    __device__ __forceinline__ explicit Cols16(const float *q)
+    {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(v[2 * k].x), "=f"(v[2 * k].y), "=f"(v[2 * k + 1].x), "=f"(v[2 * k + 1].y)
+                         : "l"(q + 4 * k));
+    }
+    __device__ __forceinline__ float2 operator[](int k) const { return v[k]; }
 };
+// the same from the constant bank or shared memory, in place
+struct Cols16Ref {
+    const float2 *p;
+    __device__ __forceinline__ explicit Cols16Ref(const float *q) : p(reinterpret_cast<const float2 *>(q)) {}
+    __device__ __forceinline__ float2 operator[](int k) const { return p[k]; }
+};
+
+// The training kernels keep the halved biases of the first two layers behind
+// their barriers in shared memory (all that is left of it); the third layer's
+// and the head's come from memory.  The operand tiles need 1024-byte alignment and leave no slack to align
+// by hand: the kernels check it.
+constexpr size_t kTrainSmem = 2 * 65536 + 3 * 32768 + 256 + 2 * kHid * sizeof(float);
+
+// Images of the training operands (activations and their gradients): per 64-row half tile its 64-column
+// blocks one after another, 64 rows x 128 bytes each, swizzled as in shared
+// memory, so a half tile is one bulk copy.  `blocks`: 4 (256 columns) or 1.
+__device__ __forceinline__ unsigned char *image_row(unsigned char *img, long long tile, int row, int block, int blocks)
+{
+    return img + (((tile * 2 + (row >> 6)) * blocks + block) << 13) + (row & 63) * 128;
+}
+constexpr long long kHalfTile = 4 * 8192;   // bytes of a 64-row half tile of 256 columns
+
+// 32 bytes (16 BF16 columns from column 16 part of a 64-column block) of row r
+// into the swizzled 128-byte row at `dst`: two 16-byte words that the swizzle
+// keeps inside one 32-byte sector, in one 32-byte store
+__device__ __forceinline__ void store_row32(unsigned char *dst, int r, int part, const uint32_t (&w)[8])
+{
+    const bool sw = r & 1;
+    unsigned char *p = dst + ((part ^ ((r >> 1) & 3)) << 5);
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(sw ? w[4] : w[0]),
+                 "r"(sw ? w[5] : w[1]), "r"(sw ? w[6] : w[2]), "r"(sw ? w[7] : w[3]), "r"(sw ? w[0] : w[4]),
+                 "r"(sw ? w[1] : w[5]), "r"(sw ? w[2] : w[6]), "r"(sw ? w[3] : w[7])
+                 : "memory");
+}
 
 // ---------------------------------------------------------------------------
 // Fused inference: features -> 3 x (tcgen05 GEMM + bias + SiLU) -> head, per
@@ -636,15 +610,29 @@ constexpr int kPairThreads = 32 * (kPairWarps + 2);      // + MMA warp + copy wa
 constexpr int kPairSlots = 3;                            // weight K-block slots
 constexpr size_t kPairSmem = 1024 + 2 * 65536 + (size_t)kPairSlots * 32768 + 256;
 
+// TRAIN (the forward pass of training): biases and head from memory (*mem),
+// where they change every step without a host round trip, instead of the
+// kernel parameters, and H1, H2 of every tile also written to the images that
+// the backward pass and the weight gradients read.
+template <bool TRAIN>
 __global__ void __launch_bounds__(kPairThreads, 1)
 k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__restrict__ lam5, long long real,
                  long long ntiles, const unsigned char *__restrict__ img1, const unsigned char *__restrict__ img2,
-                 const unsigned char *__restrict__ img3, const __grid_constant__ MlpBias bias,
-                 float *__restrict__ logit, int *err)
+                 const unsigned char *__restrict__ img3, const __grid_constant__ MlpBias val,
+                 const MlpBias *__restrict__ mem, unsigned char *__restrict__ imgH1,
+                 unsigned char *__restrict__ imgH2, float *__restrict__ logit, int *err)
 {
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char *sm = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const MlpBias &bias = TRAIN ? *mem : val;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *sm = smem_raw;
+    if constexpr (TRAIN) {
+        if (smem_u32(sm) & 1023u) {
+            if (threadIdx.x == 0) atomicExch(err, 1);
+            return;
+        }
+    } else {
+        sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    }
     unsigned char *const sH0 = sm, *const sH1 = sm + 65536;   // H of tile A, B
     unsigned char *const sW = sm + 2 * 65536;                  // weight slots
     uint64_t *bars = reinterpret_cast<uint64_t *>(sW + kPairSlots * 32768);
@@ -656,6 +644,7 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
     uint64_t *drain = bars + 18;                 // every issued MMA done
     uint64_t *partd = bars + 19;                 // [2] head partial sums of tile X written
     uint32_t *holder = reinterpret_cast<uint32_t *>(bars + 21);
+    float *sB = reinterpret_cast<float *>(bars + 32);   // TRAIN: b1, b2
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp == 0) tmem_alloc(holder, 512);
     if (tid == 0) {
@@ -672,10 +661,17 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
         mbar_init(drain, 1);
         fence_mbar_init();
     }
+    if constexpr (TRAIN) {
+        for (int i = tid; i < kHid; i += kPairThreads) {
+            sB[i] = bias.b1[i];
+            sB[kHid + i] = bias.b2[i];
+        }
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t taddr = *holder;
+    const float *const hb1 = TRAIN ? sB : bias.b1, *const hb2 = TRAIN ? sB + kHid : bias.b2;
     const long long npairs = (ntiles + 1) / 2;
     auto slot = [&](long long q) { return sW + (int)(q % kPairSlots) * 32768; };
     bool ok = true;
@@ -810,7 +806,7 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
         // epilogue of a hidden layer of tile x (bias bv): H_x chunk c, arrival c
         // (every chunk's load is waited for before the first arrival: the
         // next layer's first MMA overwrites the whole accumulator)
-        auto epilogue = [&](int x, const float *bv) {
+        auto epilogue = [&](int x, const float *bv, unsigned char *img, long long t) {
             if (!(ok && mbar_wait_warp(&accr[x], nacc[x] & 1))) return false;
             ++nacc[x];
             tc_fence_after();
@@ -821,17 +817,15 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
             for (int c = 0; c < 4; ++c) tc_ld_16cols_issue(acc + 64u * c, r[c]);
 #pragma unroll
             for (int c = 0; c < 4; ++c) tc_ld_wait16(r[c]);
-            const float2 *bv2 = reinterpret_cast<const float2 *>(bv);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const uint32_t *rc = r[c];
-                const int col0 = 64 * c + 16 * cpart;
+                const Cols16Ref b(bv + 64 * c + 16 * cpart);
                 uint32_t w[8];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const float2 y = silu_pair(make_float2(__uint_as_float(rc[2 * t]), __uint_as_float(rc[2 * t + 1])),
-                                               bv2[col0 / 2 + t]);
-                    w[t] = cvt_bf16x2(y.x, y.y);
+                for (int k = 0; k < 8; ++k) {
+                    const float2 y = silu_pair(make_float2(__uint_as_float(rc[2 * k]), __uint_as_float(rc[2 * k + 1])), b[k]);
+                    w[k] = cvt_bf16x2(y.x, y.y);
                 }
                 unsigned char *blk = H + c * 16384;
                 *reinterpret_cast<uint4 *>(blk + sw128_offset(row, 16 * cpart)) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -841,6 +835,9 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&chunk[4 * x + c]);
+                if constexpr (TRAIN) {
+                    if (t < ntiles) store_row32(image_row(img, t, row, c, 4), row, cpart, w);
+                }
             }
             return true;
         };
@@ -864,20 +861,17 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
             for (int c = 0; c < 4; ++c) tc_ld_16cols_issue(acc + 64u * c, r[c]);
 #pragma unroll
             for (int c = 0; c < 4; ++c) tc_ld_wait16(r[c]);
-            const float2 *b3 = reinterpret_cast<const float2 *>(bias.b3);
-            const float2 *w4 = reinterpret_cast<const float2 *>(bias.w4);
             float2 sum = make_float2(0.f, 0.f);   // even and odd columns
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const uint32_t *rc = r[c];
-                const int col0 = 64 * c + 16 * cpart;
+                using Cols = std::conditional_t<TRAIN, Cols16, Cols16Ref>;
+                const Cols b3(bias.b3 + 64 * c + 16 * cpart), w4(bias.w4 + 64 * c + 16 * cpart);
 #pragma unroll
-                for (int t2 = 0; t2 < 8; ++t2) {
-                    const float2 y = silu_pair(make_float2(__uint_as_float(rc[2 * t2]), __uint_as_float(rc[2 * t2 + 1])),
-                                               b3[col0 / 2 + t2]);
+                for (int k = 0; k < 8; ++k) {
+                    const float2 y = silu_pair(make_float2(__uint_as_float(rc[2 * k]), __uint_as_float(rc[2 * k + 1])), b3[k]);
                     const uint32_t hb = cvt_bf16x2(y.x, y.y);   // the activations rounded to BF16
-                    sum = fma2(make_float2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xFFFF0000u)),
-                               w4[col0 / 2 + t2], sum);
+                    sum = fma2(make_float2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xFFFF0000u)), w4[k], sum);
                 }
             }
             part[cpart * 128 + row] = sum.x + sum.y;
@@ -900,10 +894,10 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
         for (long long p = blockIdx.x; p < npairs; p += gridDim.x) {
             const long long pn = p + gridDim.x;
             const bool next = pn < npairs;
-            ok = epilogue(0, bias.b1);
-            ok = epilogue(1, bias.b1);
-            ok = epilogue(0, bias.b2);
-            ok = epilogue(1, bias.b2);
+            ok = epilogue(0, hb1, imgH1, 2 * p);
+            ok = epilogue(1, hb1, imgH1, 2 * p + 1);
+            ok = epilogue(0, hb2, imgH2, 2 * p);
+            ok = epilogue(1, hb2, imgH2, 2 * p + 1);
             ok = head(0, 2 * p, next, 2 * pn);
             ok = head(1, 2 * p + 1, next, 2 * pn + 1);
             if (!ok) break;   // (each warp on its own: no CTA-wide barrier in the loop)
@@ -918,189 +912,198 @@ k_mlp_infer_pair(RowSpec rs, const uint4 *__restrict__ ftab, const uint32_t *__r
 
 }  // namespace ens
 
+#include "ens_train.cuh"
+
 using namespace ens;
 
 // ---------------------------------------------------------------------------
 // surrogate object
 // ---------------------------------------------------------------------------
+// device memory that grows on demand and is kept for later calls
+struct Buf {
+    void *p = nullptr;
+    size_t cap = 0;
+    bool need(size_t bytes)
+    {
+        if (bytes <= cap) return true;
+        if (p) cudaFree(p);
+        p = nullptr;
+        cap = 0;
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        cap = bytes;
+        return true;
+    }
+    template <class T>
+    T *as() const { return static_cast<T *>(p); }
+    ~Buf() { if (p) cudaFree(p); }
+};
+
 struct ens_surrogate {
     cudaStream_t s = nullptr;
     ParamLayout L{};
     float *p = nullptr, *g = nullptr, *m1 = nullptr, *m2 = nullptr;
-    __nv_bfloat16 *W1b = nullptr, *W2b = nullptr, *W3b = nullptr, *W2t = nullptr, *W3t = nullptr;
     int *err = nullptr;
     long long steps = 0;
-    // work buffers for a given padded row count
-    long long cap = 0;
-    __nv_bfloat16 *X = nullptr, *Xt = nullptr, *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *H1t = nullptr,
-                  *H2t = nullptr, *dZ = nullptr, *dZt = nullptr;
-    float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *logit = nullptr, *dlogit = nullptr, *q = nullptr,
-          *target = nullptr, *dH = nullptr, *part = nullptr;
-    double *lam = nullptr, *loss = nullptr, *wq = nullptr, *pdf = nullptr;
-    uint32_t *lam5 = nullptr;   // BF16 of lambda / 5 per lambda value (fused inference)
-    int groups_cap = 0;
-    unsigned char *img = nullptr;   // swizzled W1 | W2 | W3 images for the fused inference kernel
+    double *lam = nullptr, *wq = nullptr, *pdf = nullptr;
+    uint32_t *lam5 = nullptr;       // BF16 of lambda / 5 per lambda value
+    unsigned char *img = nullptr;   // swizzled W1 | W2 | W3 images of the fused kernels
+    MlpBias *bias = nullptr;        // biases and head in device memory (with img)
+    MlpBias hbias{};                // the same on the host, valid while hbias_ok
+    bool hbias_ok = false;
     int sms = 0;
+    Buf logit, q, ftab, loss;                                  // every path
+    Buf counts, target, dlogit, images, part, head_part;       // training
+    Buf X, H, Z, Wb;                                           // layer-by-layer forward pass
 };
 
 namespace {
 
 constexpr int kMaxSplit = 32;
 
-bool alloc_work(ens_surrogate *S, long long rows, int groups)
+cudaError_t train_prepare()
 {
-    if (rows <= S->cap && groups <= S->groups_cap) return true;
-    auto fr = [&](void *p) { if (p) cudaFree(p); };
-    for (void *p : {(void *)S->X, (void *)S->Xt, (void *)S->H1, (void *)S->H2, (void *)S->H3, (void *)S->H1t,
-                    (void *)S->H2t, (void *)S->dZ, (void *)S->dZt, (void *)S->Z1, (void *)S->Z2, (void *)S->Z3,
-                    (void *)S->logit, (void *)S->dlogit, (void *)S->q, (void *)S->target, (void *)S->dH,
-                    (void *)S->part, (void *)S->lam, (void *)S->lam5, (void *)S->loss})
-        fr(p);
-    bool ok = true;
-    auto al = [&](auto **p, size_t bytes) {
-        if (cudaMalloc((void **)p, bytes) != cudaSuccess) ok = false;
-    };
-    const size_t bh = sizeof(__nv_bfloat16) * rows * kHid;
-    al(&S->X, sizeof(__nv_bfloat16) * rows * kIn);
-    al(&S->Xt, sizeof(__nv_bfloat16) * rows * kIn);
-    al(&S->H1, bh); al(&S->H2, bh); al(&S->H3, bh); al(&S->H1t, bh); al(&S->H2t, bh);
-    al(&S->dZ, bh); al(&S->dZt, bh);
-    const size_t fz = sizeof(float) * rows * kHid;
-    al(&S->Z1, fz); al(&S->Z2, fz); al(&S->Z3, fz); al(&S->dH, fz);
-    al(&S->logit, sizeof(float) * rows);
-    al(&S->dlogit, sizeof(float) * rows);
-    al(&S->q, sizeof(float) * rows);
-    al(&S->target, sizeof(float) * rows);
-    al(&S->part, sizeof(float) * kMaxSplit * kHid * kHid);
-    al(&S->lam, sizeof(double) * 4096);
-    al(&S->lam5, sizeof(uint32_t) * 4096);
-    al(&S->loss, sizeof(double) * (groups + 1));
-    S->cap = ok ? rows : 0;
-    S->groups_cap = ok ? groups : 0;
-    return ok;
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_infer_pair<false>, attr, (int)kPairSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_infer_pair<true>, attr, (int)kTrainSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_back, attr, (int)kTrainSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_wgrad, attr, (int)kWgSmem);
+    return e;
 }
 
 int blocks(long long n, int t) { return (int)((n + t - 1) / t); }
+long long pad128(long long r) { return (r + 127) / 128 * 128; }
 
-// forward through the network for `rows` padded rows of features in S->X
-bool forward(ens_surrogate *S, long long rows, bool keep_t)
+// rows' logits and densities, the feature table and the group losses
+bool alloc_rows(ens_surrogate *S, const RowSpec &rs, long long rows, int groups)
+{
+    return S->logit.need(sizeof(float) * rows) && S->q.need(sizeof(float) * rows) &&
+           S->ftab.need(sizeof(uint4) * (kIn / 8) * rs.per_member) && S->loss.need(sizeof(double) * groups);
+}
+
+// CTAs per layer of the weight-gradient kernel: one wave over the SMs, in
+// proportion to the bytes of a half tile (64 + 64 KB, 64 + 64 KB, 64 + 16 KB)
+WgradSplits wgrad_splits(const ens_surrogate *S, long long halves)
+{
+    const int sms = std::max(S->sms, 3);
+    WgradSplits sp;
+    sp.n[2] = sp.n[1] = std::max(1, sms * 8 / 21);
+    sp.n[0] = std::max(1, sms - 2 * sp.n[1]);
+    for (int &n : sp.n) n = (int)std::min<long long>(n, halves);
+    return sp;
+}
+
+TrainImages train_images(const ens_surrogate *S, long long rows)
+{
+    const size_t b = sizeof(__nv_bfloat16) * rows * kHid;
+    unsigned char *p = S->images.as<unsigned char>();
+    return TrainImages{p + 5 * b, p, p + b, p + 2 * b, p + 3 * b, p + 4 * b};
+}
+
+bool alloc_train(ens_surrogate *S, long long rows)
+{
+    const WgradSplits sp = wgrad_splits(S, rows / 64);
+    return S->target.need(sizeof(float) * rows) && S->dlogit.need(sizeof(float) * rows) &&
+           S->images.need(sizeof(__nv_bfloat16) * rows * (5 * kHid + kIn)) &&
+           S->part.need(sizeof(float) * kPartStride * (sp.n[0] + sp.n[1] + sp.n[2])) &&
+           S->head_part.need(sizeof(float) * kHeadPart * std::max(S->sms, 1));
+}
+
+// the fused kernels' operands after a change of the parameters
+void pack_params(ens_surrogate *S)
+{
+    k_pack_weights_img<<<blocks((long long)kHid * kHid, 256), 256, 0, S->s>>>(S->p, S->img, S->img + 32768,
+                                                                              S->img + 32768 + 131072, S->bias);
+    S->hbias_ok = false;
+}
+
+// layer-by-layer forward pass (one GEMM launch per layer) for `rows` padded
+// rows of the lambda values in S->lam: the check of the fused kernels
+bool forward_layers(ens_surrogate *S, const RowSpec &rs, int nlam, long long rows)
 {
     cudaStream_t s = S->s;
     const ParamLayout &L = S->L;
-    if (!gemm(S->X, kIn, S->W1b, kIn, S->Z1, kHid, (int)rows, kHid, kIn, 1, S->err, s)) return false;
-    k_bias_silu<<<blocks(rows * kHid, 256), 256, 0, s>>>(S->Z1, S->p + L.b1, rows, S->H1, keep_t ? S->H1t : nullptr);
-    if (!gemm(S->H1, kHid, S->W2b, kHid, S->Z2, kHid, (int)rows, kHid, kHid, 1, S->err, s)) return false;
-    k_bias_silu<<<blocks(rows * kHid, 256), 256, 0, s>>>(S->Z2, S->p + L.b2, rows, S->H2, keep_t ? S->H2t : nullptr);
-    if (!gemm(S->H2, kHid, S->W3b, kHid, S->Z3, kHid, (int)rows, kHid, kHid, 1, S->err, s)) return false;
-    k_bias_silu<<<blocks(rows * kHid, 256), 256, 0, s>>>(S->Z3, S->p + L.b3, rows, S->H3, nullptr);
-    k_head<<<blocks(rows * 32, 256), 256, 0, s>>>(S->H3, S->p + L.w4, S->p + L.b4, rows, S->logit);
+    if (!S->X.need(sizeof(__nv_bfloat16) * rows * kIn) || !S->H.need(sizeof(__nv_bfloat16) * rows * kHid) ||
+        !S->Z.need(sizeof(float) * rows * kHid) || !S->Wb.need(sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid)))
+        return false;
+    __nv_bfloat16 *X = S->X.as<__nv_bfloat16>(), *H = S->H.as<__nv_bfloat16>();
+    __nv_bfloat16 *W1 = S->Wb.as<__nv_bfloat16>(), *W2 = W1 + kHid * kIn, *W3 = W2 + kHid * kHid;
+    float *Z = S->Z.as<float>();
+    k_features<<<blocks(rows, 256), 256, 0, s>>>(rs, S->lam, nlam, rows, X);
+    k_pack_weights<<<blocks((long long)kHid * kHid, 256), 256, 0, s>>>(S->p, W1, W2, W3);
+    if (!gemm(X, kIn, W1, kIn, Z, kHid, (int)rows, kHid, kIn, 1, S->err, s)) return false;
+    k_bias_silu<<<blocks(rows * kHid, 256), 256, 0, s>>>(Z, S->p + L.b1, rows, H);
+    if (!gemm(H, kHid, W2, kHid, Z, kHid, (int)rows, kHid, kHid, 1, S->err, s)) return false;
+    k_bias_silu<<<blocks(rows * kHid, 256), 256, 0, s>>>(Z, S->p + L.b2, rows, H);
+    if (!gemm(H, kHid, W3, kHid, Z, kHid, (int)rows, kHid, kHid, 1, S->err, s)) return false;
+    k_bias_silu<<<blocks(rows * kHid, 256), 256, 0, s>>>(Z, S->p + L.b3, rows, H);
+    k_head<<<blocks(rows * 32, 256), 256, 0, s>>>(H, S->p + L.w4, S->p + L.b4, rows, S->logit.as<float>());
     return true;
 }
 
-// biases and head of the current parameters (host copy for the kernel parameters)
-// the fused kernel takes b / 2 for the hidden layers (exact in FP32)
-bool halve_biases(MlpBias *b)
+// feature table and lambda words of the lambda values in S->lam
+void feature_table(ens_surrogate *S, const RowSpec &rs, int nlam)
 {
-    for (int i = 0; i < kHid; ++i) {
-        b->b1[i] *= 0.5f;
-        b->b2[i] *= 0.5f;
-        b->b3[i] *= 0.5f;
-    }
-    return true;
+    k_feature_table<<<blocks(std::max(rs.per_member, nlam), 256), 256, 0, S->s>>>(rs, S->lam, nlam,
+                                                                                  S->ftab.as<uint4>(), S->lam5);
 }
 
-bool mlp_bias(ens_surrogate *S, MlpBias *b)
-{
-    const ParamLayout &L = S->L;
-    cudaStream_t s = S->s;
-    return cudaMemcpyAsync(b->b1, S->p + L.b1, sizeof(float) * kHid, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-           cudaMemcpyAsync(b->b2, S->p + L.b2, sizeof(float) * kHid, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-           cudaMemcpyAsync(b->b3, S->p + L.b3, sizeof(float) * kHid, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-           cudaMemcpyAsync(b->w4, S->p + L.w4, sizeof(float) * kHid, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-           cudaMemcpyAsync(&b->b4, S->p + L.b4, sizeof(float), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-           cudaStreamSynchronize(s) == cudaSuccess && halve_biases(b);
-}
-
-// the fused inference kernel over `real` rows of the feature table ftab
-// (one CTA per tile pair, at most one per SM)
-void launch_infer(ens_surrogate *S, const RowSpec &rs, const uint4 *ftab, long long real, const MlpBias &bias)
+// the fused forward kernel over `real` rows (one CTA per tile pair, at most
+// one per SM) into S->logit; with images: the forward pass of training
+void launch_infer(ens_surrogate *S, const RowSpec &rs, long long real, const TrainImages *im)
 {
     const long long ntiles = (real + 127) / 128;
     const int grid = (int)std::min<long long>((ntiles + 1) / 2, S->sms > 0 ? S->sms : 1);
     unsigned char *i1 = S->img, *i2 = S->img + 32768, *i3 = S->img + 32768 + 131072;
-    k_mlp_infer_pair<<<grid, kPairThreads, kPairSmem, S->s>>>(rs, ftab, S->lam5, real, ntiles, i1, i2, i3, bias,
-                                                              S->logit, S->err);
+    const uint4 *ftab = S->ftab.as<uint4>();
+    if (im)
+        k_mlp_infer_pair<true><<<grid, kPairThreads, kTrainSmem, S->s>>>(rs, ftab, S->lam5, real, ntiles, i1, i2, i3,
+                                                                        S->hbias, S->bias, im->H1, im->H2,
+                                                                        S->logit.as<float>(), S->err);
+    else
+        k_mlp_infer_pair<false><<<grid, kPairThreads, kPairSmem, S->s>>>(rs, ftab, S->lam5, real, ntiles, i1, i2, i3,
+                                                                         S->hbias, S->bias, nullptr, nullptr,
+                                                                         S->logit.as<float>(), S->err);
+}
+
+// biases and head on the host (kernel parameters of the inference kernel)
+bool host_bias(ens_surrogate *S)
+{
+    if (S->hbias_ok) return true;
+    S->hbias_ok = cudaMemcpyAsync(&S->hbias, S->bias, sizeof(MlpBias), cudaMemcpyDeviceToHost, S->s) == cudaSuccess &&
+                  cudaStreamSynchronize(S->s) == cudaSuccess;
+    return S->hbias_ok;
 }
 
 // fused inference of `real` rows (lambda values in S->lam) into S->logit
 bool forward_fused(ens_surrogate *S, const RowSpec &rs, long long real)
 {
-    cudaStream_t s = S->s;
-    const long long n = (long long)kHid * kHid;
-    MlpBias bias;
-    if (!mlp_bias(S, &bias)) return false;
-    k_pack_weights_img<<<blocks(n, 256), 256, 0, s>>>(S->p, S->img, S->img + 32768, S->img + 32768 + 131072);
-    const int nlam = (int)(real / rs.per_member);
-    uint4 *ftab = reinterpret_cast<uint4 *>(S->Xt);   // the training path's transposed features: free here
-    k_feature_table<<<blocks(std::max(rs.per_member, nlam), 256), 256, 0, s>>>(rs, S->lam, nlam, ftab, S->lam5);
-    launch_infer(S, rs, ftab, real, bias);
+    if (!host_bias(S)) return false;
+    feature_table(S, rs, (int)(real / rs.per_member));
+    launch_infer(S, rs, real, nullptr);
     return cudaGetLastError() == cudaSuccess;
 }
 
-int pick_split(long long rows)
-{
-    int sp = kMaxSplit;
-    while (sp > 1 && (rows % (64LL * sp) != 0 || rows / sp < 512)) --sp;
-    return sp;
-}
-
-// backward pass into S->g (gradients of the mean group loss)
-bool backward(ens_surrogate *S, long long rows, long long real)
+// loss (loss null: not wanted) and gradient of the batch in S->lam, S->target
+void loss_grad_kernels(ens_surrogate *S, const RowSpec &rs, int n, long long rows, long long real, bool want_loss)
 {
     cudaStream_t s = S->s;
-    const ParamLayout &L = S->L;
-    k_head_grad<<<kHid + 1, 256, 0, s>>>(S->dlogit, S->H3, real, S->g + L.w4, S->g + L.b4);
-    k_head_back<<<blocks(rows * kHid, 256), 256, 0, s>>>(S->dlogit, S->p + L.w4, S->Z3, rows, real, S->dZ, S->dZt);
-    const int sp = pick_split(rows);
-    // layer 3: dW3 = dZ3^T H2, db3, dH2 = dZ3 W3
-    if (!gemm(S->dZt, (int)rows, S->H2t, (int)rows, S->part, kHid, kHid, kHid, (int)rows, sp, S->err, s)) return false;
-    k_sum_splits<<<blocks((long long)kHid * kHid, 256), 256, 0, s>>>(S->part, sp, (long long)kHid * kHid, S->g + L.W3);
-    k_colsum_bf16<<<kHid, 256, 0, s>>>(S->dZ, rows, S->g + L.b3);
-    if (!gemm(S->dZ, kHid, S->W3t, kHid, S->dH, kHid, (int)rows, kHid, kHid, 1, S->err, s)) return false;
-    k_silu_back<<<blocks(rows * kHid, 256), 256, 0, s>>>(S->dH, S->Z2, rows, S->dZ, S->dZt);
-    // layer 2
-    if (!gemm(S->dZt, (int)rows, S->H1t, (int)rows, S->part, kHid, kHid, kHid, (int)rows, sp, S->err, s)) return false;
-    k_sum_splits<<<blocks((long long)kHid * kHid, 256), 256, 0, s>>>(S->part, sp, (long long)kHid * kHid, S->g + L.W2);
-    k_colsum_bf16<<<kHid, 256, 0, s>>>(S->dZ, rows, S->g + L.b2);
-    if (!gemm(S->dZ, kHid, S->W2t, kHid, S->dH, kHid, (int)rows, kHid, kHid, 1, S->err, s)) return false;
-    k_silu_back<<<blocks(rows * kHid, 256), 256, 0, s>>>(S->dH, S->Z1, rows, S->dZ, S->dZt);
-    // layer 1: dW1 = dZ1^T X (N = 64)
-    if (!gemm(S->dZt, (int)rows, S->Xt, (int)rows, S->part, kIn, kHid, kIn, (int)rows, sp, S->err, s)) return false;
-    k_sum_splits<<<blocks((long long)kHid * kIn, 256), 256, 0, s>>>(S->part, sp, (long long)kHid * kIn, S->g + L.W1);
-    k_colsum_bf16<<<kHid, 256, 0, s>>>(S->dZ, rows, S->g + L.b1);
-    return true;
-}
-
-long long pad128(long long r) { return (r + 127) / 128 * 128; }
-
-// targets: normalised in-range histograms of each member and kind
-void make_targets(int n, const uint64_t *counts, const ens_hist_spec *h, std::vector<float> &t)
-{
-    const int nq = h->qr_bins, nt = h->tail_bins;
-    const int per = nq * nq + 2 * nt;
-    const long long L = counts_len_of(nq, nt, h->grad_bins);
-    t.assign((size_t)n * per, 0.f);
-    for (int i = 0; i < n; ++i) {
-        const uint64_t *c = counts + (size_t)i * L;
-        const int off[3] = {0, nq * nq, nq * nq + nt};
-        const int len[3] = {nq * nq, nt, nt};
-        for (int k = 0; k < 3; ++k) {
-            double s = 0.0;
-            for (int b = 0; b < len[k]; ++b) s += (double)c[off[k] + b];
-            for (int b = 0; b < len[k]; ++b)
-                t[(size_t)i * per + off[k] + b] = s > 0.0 ? (float)((double)c[off[k] + b] / s) : 0.f;
-        }
-    }
+    const double wgt = 1.0 / (3.0 * n);
+    const TrainImages im = train_images(S, rows);
+    launch_infer(S, rs, real, &im);
+    // one wave of large groups: 1024 threads each
+    k_softmax_ce<<<3 * n, 1024, 0, s>>>(S->logit.as<float>(), S->target.as<float>(), rs.nq, rs.nt, wgt, nullptr,
+                                       S->dlogit.as<float>(), want_loss ? S->loss.as<double>() : nullptr);
+    const long long ntiles = rows / 128;
+    const int grid = (int)std::min<long long>(ntiles, S->sms > 0 ? S->sms : 1);
+    k_mlp_back<<<grid, kPairThreads, kTrainSmem, s>>>(rs, S->ftab.as<uint4>(), S->lam5, real, ntiles, S->img,
+                                                     S->img + 32768, S->img + 32768 + 131072, S->bias,
+                                                     S->dlogit.as<float>(), im, S->head_part.as<float>(), S->err);
+    const WgradSplits sp = wgrad_splits(S, rows / 64);
+    k_mlp_wgrad<<<sp.n[0] + sp.n[1] + sp.n[2], kWgThreads, kWgSmem, s>>>(im, rows / 64, sp, S->part.as<float>(), S->err);
+    k_grad_sum<<<blocks(S->L.total, 256), 256, 0, s>>>(S->part.as<float>(), sp, S->head_part.as<float>(), grid, S->g);
 }
 
 }  // namespace
@@ -1118,30 +1121,27 @@ ens_status ens_surrogate_create(uint64_t seed, void *stream, ens_surrogate **out
     bool ok = gemm_prepare() == cudaSuccess;
     ok = ok && cudaMalloc(&S->p, sizeof(float) * n) == cudaSuccess && cudaMalloc(&S->g, sizeof(float) * n) == cudaSuccess &&
          cudaMalloc(&S->m1, sizeof(float) * n) == cudaSuccess && cudaMalloc(&S->m2, sizeof(float) * n) == cudaSuccess &&
-         cudaMalloc(&S->W1b, sizeof(__nv_bfloat16) * kHid * kIn) == cudaSuccess &&
-         cudaMalloc(&S->W2b, sizeof(__nv_bfloat16) * kHid * kHid) == cudaSuccess &&
-         cudaMalloc(&S->W3b, sizeof(__nv_bfloat16) * kHid * kHid) == cudaSuccess &&
-         cudaMalloc(&S->W2t, sizeof(__nv_bfloat16) * kHid * kHid) == cudaSuccess &&
-         cudaMalloc(&S->W3t, sizeof(__nv_bfloat16) * kHid * kHid) == cudaSuccess &&
+         cudaMalloc(&S->lam, sizeof(double) * 4096) == cudaSuccess &&
+         cudaMalloc(&S->lam5, sizeof(uint32_t) * 4096) == cudaSuccess &&
+         cudaMalloc(&S->bias, sizeof(MlpBias)) == cudaSuccess &&
          cudaMalloc(&S->err, sizeof(int)) == cudaSuccess && cudaMalloc(&S->wq, sizeof(double) * 4096) == cudaSuccess &&
          cudaMalloc(&S->pdf, sizeof(double) * 1 << 20) == cudaSuccess &&
          cudaMalloc(&S->img, 32768 + 2 * 131072) == cudaSuccess &&
-         cudaFuncSetAttribute(k_mlp_infer_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem) ==
-             cudaSuccess;
+         train_prepare() == cudaSuccess;
     int dev = 0;
     ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
          cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
     if (!ok) {
-        delete S;
+        ens_surrogate_destroy(S);
         return ENS_ENOMEM;
     }
     cudaMemsetAsync(S->err, 0, sizeof(int), S->s);
     cudaMemsetAsync(S->m1, 0, sizeof(float) * n, S->s);
     cudaMemsetAsync(S->m2, 0, sizeof(float) * n, S->s);
     k_init_params<<<blocks(n, 256), 256, 0, S->s>>>(S->p, n, seed);
-    k_pack_weights<<<blocks((long long)kHid * kHid, 256), 256, 0, S->s>>>(S->p, S->W1b, S->W2b, S->W3b, S->W2t, S->W3t);
+    pack_params(S);
     if (cudaStreamSynchronize(S->s) != cudaSuccess) {
-        delete S;
+        ens_surrogate_destroy(S);
         return ENS_ECUDA;
     }
     *out = S;
@@ -1152,13 +1152,8 @@ ens_status ens_surrogate_destroy(ens_surrogate *S)
 {
     if (!S) return ENS_EINVAL;
     cudaStreamSynchronize(S->s);
-    for (void *p : {(void *)S->p, (void *)S->g, (void *)S->m1, (void *)S->m2, (void *)S->W1b, (void *)S->W2b,
-                    (void *)S->W3b, (void *)S->W2t, (void *)S->W3t, (void *)S->err, (void *)S->wq, (void *)S->pdf,
-                    (void *)S->img,
-                    (void *)S->X, (void *)S->Xt, (void *)S->H1, (void *)S->H2, (void *)S->H3, (void *)S->H1t,
-                    (void *)S->H2t, (void *)S->dZ, (void *)S->dZt, (void *)S->Z1, (void *)S->Z2, (void *)S->Z3,
-                    (void *)S->logit, (void *)S->dlogit, (void *)S->q, (void *)S->target, (void *)S->dH,
-                    (void *)S->part, (void *)S->lam, (void *)S->lam5, (void *)S->loss})
+    for (void *p : {(void *)S->p, (void *)S->g, (void *)S->m1, (void *)S->m2, (void *)S->err, (void *)S->wq,
+                    (void *)S->pdf, (void *)S->img, (void *)S->bias, (void *)S->lam, (void *)S->lam5})
         if (p) cudaFree(p);
     delete S;
     return ENS_OK;
@@ -1180,11 +1175,12 @@ ens_status ens_surrogate_set_params(ens_surrogate *S, const float *host)
     if (!S || !host) return ENS_EINVAL;
     if (cudaMemcpyAsync(S->p, host, sizeof(float) * S->L.total, cudaMemcpyHostToDevice, S->s) != cudaSuccess)
         return ENS_ECUDA;
-    k_pack_weights<<<blocks((long long)kHid * kHid, 256), 256, 0, S->s>>>(S->p, S->W1b, S->W2b, S->W3b, S->W2t, S->W3t);
+    pack_params(S);
     if (cudaStreamSynchronize(S->s) != cudaSuccess) return ENS_ECUDA;
     return ENS_OK;
 }
 
+// rows and lambda values of a call; with counts, the training targets too
 static ens_status load_batch(ens_surrogate *S, int n, const double *lambdas, const uint64_t *counts,
                              const ens_hist_spec *h, long long *rows_pad, long long *real, RowSpec *rs)
 {
@@ -1194,18 +1190,16 @@ static ens_status load_batch(ens_surrogate *S, int n, const double *lambdas, con
     rs->per_member = h->qr_bins * h->qr_bins + 2 * h->tail_bins;
     *real = (long long)n * rs->per_member;
     *rows_pad = pad128(*real);
-    if (*rows_pad % 64 != 0) return ENS_EINVAL;
-    if (!alloc_work(S, *rows_pad, 3 * n)) return ENS_ENOMEM;
+    if (!alloc_rows(S, *rs, *rows_pad, 3 * n)) return ENS_ENOMEM;
     if (cudaMemcpyAsync(S->lam, lambdas, sizeof(double) * n, cudaMemcpyHostToDevice, S->s) != cudaSuccess)
         return ENS_ECUDA;
-    k_features<<<blocks(*rows_pad, 256), 256, 0, S->s>>>(*rs, S->lam, n, *rows_pad, S->X, S->Xt);
     if (counts) {
-        std::vector<float> t;
-        make_targets(n, counts, h, t);
-        if (cudaMemcpyAsync(S->target, t.data(), sizeof(float) * t.size(), cudaMemcpyHostToDevice, S->s) !=
-            cudaSuccess ||
-            cudaStreamSynchronize(S->s) != cudaSuccess)
+        const long long L = counts_len_of(h->qr_bins, h->tail_bins, h->grad_bins);
+        if (!alloc_train(S, *rows_pad) || !S->counts.need(sizeof(uint64_t) * n * L)) return ENS_ENOMEM;
+        if (cudaMemcpyAsync(S->counts.p, counts, sizeof(uint64_t) * n * L, cudaMemcpyHostToDevice, S->s) != cudaSuccess)
             return ENS_ECUDA;
+        k_targets<<<dim3(target_parts(rs->nq, rs->nt), n), 256, 0, S->s>>>(S->counts.as<unsigned long long>(), L, rs->nq, rs->nt, S->target.as<float>());
+        feature_table(S, *rs, n);
     }
     return ENS_OK;
 }
@@ -1227,14 +1221,10 @@ ens_status ens_surrogate_loss_grad(ens_surrogate *S, int n, const double *lambda
     if (!counts) return ENS_EINVAL;
     ens_status st = load_batch(S, n, lambdas, counts, h, &rows, &real, &rs);
     if (st != ENS_OK) return st;
-    const double wgt = 1.0 / (3.0 * n);
-    if (!forward(S, rows, true)) return ENS_EINVAL;
-    cudaMemsetAsync(S->dlogit, 0, sizeof(float) * rows, S->s);
-    k_softmax_ce<<<3 * n, 256, 0, S->s>>>(S->logit, S->target, rs.nq, rs.nt, wgt, S->q, S->dlogit, S->loss);
-    if (!backward(S, rows, real)) return ENS_EINVAL;
+    loss_grad_kernels(S, rs, n, rows, real, true);
     if (cudaGetLastError() != cudaSuccess) return ENS_ECUDA;
     std::vector<double> lp(3 * n);
-    if (cudaMemcpyAsync(lp.data(), S->loss, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
+    if (cudaMemcpyAsync(lp.data(), S->loss.p, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
         return ENS_ECUDA;
     if (grad_host &&
         cudaMemcpyAsync(grad_host, S->g, sizeof(float) * S->L.total, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
@@ -1257,28 +1247,23 @@ ens_status ens_surrogate_train(ens_surrogate *S, int n, const double *lambdas, c
     if (!counts || steps < 0 || !(lr > 0.0)) return ENS_EINVAL;
     ens_status st = load_batch(S, n, lambdas, counts, h, &rows, &real, &rs);
     if (st != ENS_OK) return st;
-    const double wgt = 1.0 / (3.0 * n);
     const long long np = S->L.total;
     for (int it = 0; it < steps; ++it) {
-        if (!forward(S, rows, true)) return ENS_EINVAL;
-        k_softmax_ce<<<3 * n, 256, 0, S->s>>>(S->logit, S->target, rs.nq, rs.nt, wgt, nullptr, S->dlogit,
-                                             it == steps - 1 ? S->loss : nullptr);
-        if (!backward(S, rows, real)) return ENS_EINVAL;
+        loss_grad_kernels(S, rs, n, rows, real, it == steps - 1);
         S->steps += 1;
         const float b1 = 0.9f, b2 = 0.999f;
         const float bc1 = 1.f - powf(b1, (float)S->steps), bc2 = 1.f - powf(b2, (float)S->steps);
         // cosine decay over the call's steps, from lr to lr / 20
         const double lr_t = lr * (0.05 + 0.95 * 0.5 * (1.0 + std::cos(3.14159265358979323846 * it / steps)));
         k_adam<<<blocks(np, 256), 256, 0, S->s>>>(S->p, S->g, S->m1, S->m2, np, (float)lr_t, b1, b2, 1e-8f, bc1, bc2);
-        k_pack_weights<<<blocks((long long)kHid * kHid, 256), 256, 0, S->s>>>(S->p, S->W1b, S->W2b, S->W3b, S->W2t,
-                                                                             S->W3t);
+        pack_params(S);
     }
     if (cudaGetLastError() != cudaSuccess) return ENS_ECUDA;
     st = check_err(S);
     if (st != ENS_OK) return st;
     if (final_loss && steps > 0) {
         std::vector<double> lp(3 * n);
-        if (cudaMemcpyAsync(lp.data(), S->loss, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, S->s) != cudaSuccess ||
+        if (cudaMemcpyAsync(lp.data(), S->loss.p, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, S->s) != cudaSuccess ||
             cudaStreamSynchronize(S->s) != cudaSuccess)
             return ENS_ECUDA;
         double t = 0.0;
@@ -1296,10 +1281,11 @@ ens_status ens_surrogate_density(ens_surrogate *S, int n, const double *lambdas,
     ens_status st = load_batch(S, n, lambdas, nullptr, h, &rows, &real, &rs);
     if (st != ENS_OK) return st;
     if (!forward_fused(S, rs, real)) return ENS_ECUDA;
-    k_softmax_ce<<<3 * n, 256, 0, S->s>>>(S->logit, nullptr, rs.nq, rs.nt, 1.0, S->q, nullptr, nullptr);
+    k_softmax_ce<<<3 * n, 256, 0, S->s>>>(S->logit.as<float>(), nullptr, rs.nq, rs.nt, 1.0, S->q.as<float>(), nullptr,
+                                         nullptr);
     if (cudaGetLastError() != cudaSuccess) return ENS_ECUDA;
     std::vector<float> q((size_t)real);
-    if (cudaMemcpyAsync(q.data(), S->q, sizeof(float) * real, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
+    if (cudaMemcpyAsync(q.data(), S->q.p, sizeof(float) * real, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
         return ENS_ECUDA;
     st = check_err(S);
     if (st != ENS_OK) return st;
@@ -1315,13 +1301,14 @@ ens_status ens_surrogate_mixture(ens_surrogate *S, const ens_hist_spec *h, const
     RowSpec rs{h->qr_bins, h->tail_bins, h->qr_bins * h->qr_bins + 2 * h->tail_bins};
     const long long real = (long long)nquad * rs.per_member, rows = pad128(real);
     if (rs.per_member > (1 << 20)) return ENS_EINVAL;
-    if (!alloc_work(S, rows, 3 * nquad)) return ENS_ENOMEM;
+    if (!alloc_rows(S, rs, rows, 3 * nquad)) return ENS_ENOMEM;
     k_quad_weights<<<1, 256, 0, S->s>>>(lam_lo, lam_hi, nquad, w->kind, w->c, w->Z, w->mu, w->sigma, S->lam, S->wq);
     if (!forward_fused(S, rs, real)) return ENS_ECUDA;
-    k_softmax_ce<<<3 * nquad, 256, 0, S->s>>>(S->logit, nullptr, rs.nq, rs.nt, 1.0, S->q, nullptr, nullptr);
+    k_softmax_ce<<<3 * nquad, 256, 0, S->s>>>(S->logit.as<float>(), nullptr, rs.nq, rs.nt, 1.0, S->q.as<float>(),
+                                             nullptr, nullptr);
     const double dq = 2.0 * h->q_lim / h->qr_bins, dr = 2.0 * h->r_lim / h->qr_bins;
     const double dt = (h->tail_hi - h->tail_lo) / h->tail_bins;
-    k_quad_mix<<<blocks(rs.per_member, 256), 256, 0, S->s>>>(S->q, S->wq, nquad, rs.per_member, rs.nq, dq, dr, dt,
+    k_quad_mix<<<blocks(rs.per_member, 256), 256, 0, S->s>>>(S->q.as<float>(), S->wq, nquad, rs.per_member, rs.nq, dq, dr, dt,
                                                              S->pdf);
     if (cudaGetLastError() != cudaSuccess) return ENS_ECUDA;
     std::vector<double> pdf(rs.per_member);
@@ -1344,14 +1331,19 @@ ens_status ens_surrogate_time_gemm(ens_surrogate *S, long long rows, int iters, 
 {
     if (!S || rows <= 0 || iters < 1 || !ms) return ENS_EINVAL;
     rows = pad128(rows);
-    if (!alloc_work(S, rows, 3)) return ENS_ENOMEM;
-    cudaMemsetAsync(S->H1, 0, sizeof(__nv_bfloat16) * rows * kHid, S->s);
+    if (!S->H.need(sizeof(__nv_bfloat16) * rows * kHid) || !S->Z.need(sizeof(float) * rows * kHid) ||
+        !S->Wb.need(sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid)))
+        return ENS_ENOMEM;
+    cudaMemsetAsync(S->H.p, 0, sizeof(__nv_bfloat16) * rows * kHid, S->s);
+    cudaMemsetAsync(S->Wb.p, 0, sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid), S->s);
+    const __nv_bfloat16 *H = S->H.as<__nv_bfloat16>(), *W = S->Wb.as<__nv_bfloat16>() + kHid * kIn;
+    auto launch = [&]() { gemm(H, kHid, W, kHid, S->Z.as<float>(), kHid, (int)rows, kHid, kHid, 1, S->err, S->s); };
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
-    gemm(S->H1, kHid, S->W2b, kHid, S->Z2, kHid, (int)rows, kHid, kHid, 1, S->err, S->s);   // warm-up
+    launch();   // warm-up
     cudaEventRecord(a, S->s);
-    for (int i = 0; i < iters; ++i) gemm(S->H1, kHid, S->W2b, kHid, S->Z2, kHid, (int)rows, kHid, kHid, 1, S->err, S->s);
+    for (int i = 0; i < iters; ++i) launch();
     cudaEventRecord(b, S->s);
     float t = 0.f;
     const cudaError_t e = cudaEventSynchronize(b);
@@ -1364,7 +1356,7 @@ ens_status ens_surrogate_time_gemm(ens_surrogate *S, long long rows, int iters, 
 }
 
 // logits of the network at n lambda values, by the fused inference kernel
-// (fused != 0) or by the layer-by-layer training forward pass (tests)
+// (fused != 0) or by the layer-by-layer forward pass (tests)
 ens_status ens_surrogate_logits(ens_surrogate *S, int n, const double *lambdas, const ens_hist_spec *h, int fused,
                                 float *logits)
 {
@@ -1373,8 +1365,8 @@ ens_status ens_surrogate_logits(ens_surrogate *S, int n, const double *lambdas, 
     if (!logits) return ENS_EINVAL;
     ens_status st = load_batch(S, n, lambdas, nullptr, h, &rows, &real, &rs);
     if (st != ENS_OK) return st;
-    if (fused ? !forward_fused(S, rs, real) : !forward(S, rows, false)) return ENS_ECUDA;
-    if (cudaMemcpyAsync(logits, S->logit, sizeof(float) * real, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
+    if (fused ? !forward_fused(S, rs, real) : !forward_layers(S, rs, n, rows)) return ENS_ECUDA;
+    if (cudaMemcpyAsync(logits, S->logit.p, sizeof(float) * real, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
         return ENS_ECUDA;
     return check_err(S);
 }
@@ -1386,15 +1378,11 @@ ens_status ens_surrogate_time_infer(ens_surrogate *S, const ens_hist_spec *h, in
     if (!S || !h || nquad < 1 || nquad > 4096 || iters < 1 || !ms) return ENS_EINVAL;
     RowSpec rs{h->qr_bins, h->tail_bins, h->qr_bins * h->qr_bins + 2 * h->tail_bins};
     const long long real = (long long)nquad * rs.per_member, rows = pad128(real);
-    if (!alloc_work(S, rows, 3 * nquad)) return ENS_ENOMEM;
+    if (!alloc_rows(S, rs, rows, 3 * nquad)) return ENS_ENOMEM;
     k_quad_weights<<<1, 256, 0, S->s>>>(-5.0, 5.0, nquad, 1, 0.0, 0.0, 0.0, 1.0, S->lam, S->wq);
-    k_pack_weights_img<<<blocks((long long)kHid * kHid, 256), 256, 0, S->s>>>(S->p, S->img, S->img + 32768,
-                                                                              S->img + 32768 + 131072);
-    MlpBias bias;
-    if (!mlp_bias(S, &bias)) return ENS_ECUDA;
-    uint4 *ftab = reinterpret_cast<uint4 *>(S->Xt);
-    k_feature_table<<<blocks(std::max(rs.per_member, nquad), 256), 256, 0, S->s>>>(rs, S->lam, nquad, ftab, S->lam5);
-    auto launch = [&]() { launch_infer(S, rs, ftab, real, bias); };
+    if (!host_bias(S)) return ENS_ECUDA;
+    feature_table(S, rs, nquad);
+    auto launch = [&]() { launch_infer(S, rs, real, nullptr); };
     launch();   // warm-up
     cudaEvent_t a, b;
     cudaEventCreate(&a);

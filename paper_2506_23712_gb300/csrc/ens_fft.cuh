@@ -153,14 +153,33 @@ __device__ __forceinline__ float2 twmul(float2 a)
     }
 }
 
+// every second bit of a slot mask, from bit `odd` on
+__host__ __device__ constexpr unsigned half_mask(unsigned m, int odd)
+{
+    unsigned r = 0;
+    for (int i = 0; i < 16; ++i) r |= ((m >> (2 * i + odd)) & 1u) << i;
+    return r;
+}
+
 // In-register R-point DFT, natural order in and out; PK: packed FP32x2
-// complex adds.
-template <int R, bool FWD, bool PK = false>
+// complex adds.  ZM: inputs known to be zero (bit i: v[i]); a half whose
+// inputs are all zero costs no butterfly (x + 0 is x, so the results are the
+// same), which the compiler may not do by itself for floating-point zeros.
+template <int R, bool FWD, bool PK = false, unsigned ZM = 0u>
 struct Dft {
+    static constexpr unsigned ALL = (1u << (R / 2)) - 1u, ZE = half_mask(ZM, 0), ZO = half_mask(ZM, 1);
     template <int K>
     static __device__ __forceinline__ void combine(float2 *v, const float2 *e, const float2 *o)
     {
-        if constexpr (K < R / 2) {
+        if constexpr (K < R / 2 && ZO == ALL) {
+            v[K] = v[K + R / 2] = e[K];
+            combine<K + 1>(v, e, o);
+        } else if constexpr (K < R / 2 && ZE == ALL) {
+            const float2 t = twmul<R, K, FWD>(o[K]);
+            v[K] = t;
+            v[K + R / 2] = make_float2(-t.x, -t.y);
+            combine<K + 1>(v, e, o);
+        } else if constexpr (K < R / 2) {
             constexpr int j = (K * (48 / R)) % 48;
             if constexpr (j % 12 == 6) {
                 // W = h (sc + i ss) with h = sqrt(2)/2: o W = h (A + i B), and
@@ -195,29 +214,36 @@ struct Dft {
             e[i] = v[2 * i];
             o[i] = v[2 * i + 1];
         }
-        Dft<H, FWD, PK>::run(e);
-        Dft<H, FWD, PK>::run(o);
+        Dft<H, FWD, PK, ZE>::run(e);
+        Dft<H, FWD, PK, ZO>::run(o);
         combine<0>(v, e, o);
     }
 };
 
-template <bool FWD, bool PK>
-struct Dft<1, FWD, PK> {
+template <bool FWD, bool PK, unsigned ZM>
+struct Dft<1, FWD, PK, ZM> {
     static __device__ __forceinline__ void run(float2 *) {}
 };
 
-template <bool FWD, bool PK>
-struct Dft<2, FWD, PK> {
+template <bool FWD, bool PK, unsigned ZM>
+struct Dft<2, FWD, PK, ZM> {
     static __device__ __forceinline__ void run(float2 *v)
     {
         const float2 a = v[0], b = v[1];
-        v[0] = cadd_<PK>(a, b);
-        v[1] = csub_<PK>(a, b);
+        if constexpr (ZM == 0u) {
+            v[0] = cadd_<PK>(a, b);
+            v[1] = csub_<PK>(a, b);
+        } else if constexpr (ZM == 1u) {
+            v[0] = b;
+            v[1] = make_float2(-b.x, -b.y);
+        } else {   // b (or both) zero
+            v[1] = a;
+        }
     }
 };
 
-template <bool FWD, bool PK>
-struct Dft<3, FWD, PK> {
+template <bool FWD, bool PK, unsigned ZM>
+struct Dft<3, FWD, PK, ZM> {
     static __device__ __forceinline__ void run(float2 *v)
     {
         // X1,2 = v0 - (v1+v2)/2 -/+ s i (sqrt3/2)(v1 - v2), s = +1 fwd
@@ -332,20 +358,148 @@ __device__ __forceinline__ void exchange(float2 *v, int p, At at, Sync sync = Sy
     }
 }
 
+// Inter-pass twiddles of a column plan in shared memory: the pass of radix R
+// after Ns points multiplies slot t of the butterfly with k = j mod Ns by
+// W_N^(t k N / (Ns R)); entry (t - 1) Ns + k of the pass's table, so a thread
+// reads them at one base plus compile-time offsets (indexing the N-entry table
+// by t k costs an address per value).  N - R0 entries in all.
+template <int N, int VAR>
+struct ColTw {
+    using PI = PlanInfo<N, VAR>;
+    static constexpr int R0 = PI::R0, R1 = PI::R1, R2 = PI::R2;
+    static constexpr int OFF2 = (R1 - 1) * R0, SIZE = N - R0;
+    // whole block (TH threads from `tid`); no barrier
+    static __device__ __forceinline__ void load(float2 *tab, const float2 *__restrict__ g, int tid, int TH)
+    {
+        for (int i = tid; i < SIZE; i += TH) {
+            const bool second = PI::NP == 3 && i >= OFF2;
+            const int j = second ? i - OFF2 : i, Ns = second ? R0 * R1 : R0, R = second ? R2 : R1;
+            tab[i] = g[(j / Ns + 1) * (j % Ns) * (N / (Ns * R))];
+        }
+    }
+};
+
+// a pass after Ns points, its twiddles from a ColTw table
+template <int N, int R, int Ns, int P, bool FWD, bool PK>
+__device__ __forceinline__ void pass_regs_ct(float2 *v, int p, const float2 *__restrict__ tab)
+{
+    constexpr int B = N / (R * P);
+    static_assert(P % Ns == 0 || (Ns % P == 0 && B * P <= Ns), "butterflies of a thread share k or continue it");
+    const float2 *t0 = tab + (P % Ns == 0 ? p % Ns : p);
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+#pragma unroll
+        for (int t = 1; t < R; ++t) {
+            float2 w = t0[(t - 1) * Ns + (P % Ns == 0 ? 0 : b * P)];
+            if (!FWD) w.y = -w.y;
+            v[b * R + t] = cmul(v[b * R + t], w);
+        }
+        Dft<R, FWD, PK>::run(&v[b * R]);
+    }
+}
+
+// Register slots of a pruned column line.  Slot i of thread p holds position
+// p + c of the line, c known at compile time: in(i) before the first pass,
+// out(i) after the last.  Whether the 2/3 rule keeps it follows from c but for
+// the two slots that straddle the limits; row(c) + p is its row in the
+// compact layout.
+template <int N, int VAR>
+struct ColSlots {
+    using PI = PlanInfo<N, VAR>;
+    static constexpr int P = PI::P, V = PI::V, KC = (N + 2) / 3 - 1, NK = 2 * KC + 1;
+    enum Kind { kLow, kLowMixed, kZero, kNegMixed, kNeg };
+    static __host__ __device__ constexpr int in(int i) { return (i / PI::R0) * P + (i % PI::R0) * (N / PI::R0); }
+    static __host__ __device__ constexpr int out(int i) { return (i / PI::RL) * P + (i % PI::RL) * (N / PI::RL); }
+    static __host__ __device__ constexpr Kind kind(int c)
+    {
+        return c + P - 1 <= KC ? kLow : c >= N - KC ? kNeg : c > KC && c + P - 1 < N - KC ? kZero : c <= KC ? kLowMixed : kNegMixed;
+    }
+    static_assert(P <= N - 2 * KC - 1, "a slot meets one limit at most");
+    static __host__ __device__ constexpr int row(int c) { return c <= KC ? c : c + NK - N; }
+    static __host__ __device__ constexpr int wave(int c) { return c <= KC ? c : c - N; }   // wave number - p
+    // first-pass inputs of butterfly b that are zero for every thread
+    static __host__ __device__ constexpr unsigned zeros(int b)
+    {
+        unsigned m = 0;
+        for (int t = 0; t < PI::R0; ++t)
+            if (kind(in(b * PI::R0 + t)) == kZero) m |= 1u << t;
+        return m;
+    }
+};
+
+template <int C>
+struct Int {
+    static constexpr int value = C;
+};
+
+// for every kept input slot: v[I] = f(Int<c>), zero elsewhere (and for !valid)
+template <int N, int VAR, int I = 0, class F>
+__device__ __forceinline__ void load_kept(float2 *v, int p, bool valid, F f)
+{
+    using CS = ColSlots<N, VAR>;
+    if constexpr (I < CS::V) {
+        constexpr int c = CS::in(I);
+        constexpr auto k = CS::kind(c);
+        bool keep = valid;
+        if constexpr (k == CS::kLowMixed) keep = keep && p <= CS::KC - c;
+        if constexpr (k == CS::kNegMixed) keep = keep && p >= N - CS::KC - c;
+        if constexpr (k == CS::kZero) {
+            v[I] = make_float2(0.f, 0.f);
+        } else {
+            v[I] = make_float2(0.f, 0.f);
+            if (keep) v[I] = f(Int<c>());
+        }
+        load_kept<N, VAR, I + 1>(v, p, valid, f);
+    }
+}
+
+// for every kept output slot: f(Int<c>, v[I])
+template <int N, int VAR, int I = 0, class F>
+__device__ __forceinline__ void store_kept(const float2 *v, int p, bool valid, F f)
+{
+    using CS = ColSlots<N, VAR>;
+    if constexpr (I < CS::V) {
+        constexpr int c = CS::out(I);
+        constexpr auto k = CS::kind(c);
+        if constexpr (k != CS::kZero) {
+            bool keep = valid;
+            if constexpr (k == CS::kLowMixed) keep = keep && p <= CS::KC - c;
+            if constexpr (k == CS::kNegMixed) keep = keep && p >= N - CS::KC - c;
+            if (keep) f(Int<c>(), v[I]);
+        }
+        store_kept<N, VAR, I + 1>(v, p, valid, f);
+    }
+}
+
+// first pass of a column line; PRUNED: the zero band's inputs are zero
+template <int N, bool FWD, int VAR, bool PK, bool PRUNED, int B = 0>
+__device__ __forceinline__ void first_pass(float2 *v)
+{
+    using PI = PlanInfo<N, VAR>;
+    if constexpr (B < PI::V / PI::R0) {
+        Dft<PI::R0, FWD, PK, PRUNED ? ColSlots<N, VAR>::zeros(B) : 0u>::run(&v[B * PI::R0]);
+        first_pass<N, FWD, VAR, PK, PRUNED, B + 1>(v);
+    }
+}
+
 // Full line transform.  In: v in first-pass input order.  Out: v in
 // last-pass output order (PlanInfo::out_pos).  Every thread of the block (of
-// the group, with a NamedSync) must call it: it contains barriers.
-template <int N, bool FWD, int VAR = 0, class At, class Sync = BlockSync>
-__device__ __forceinline__ void fft_line(float2 *v, int p, const float2 *__restrict__ tw, At at, Sync sync = Sync())
+// the group, with a NamedSync) must call it: it contains barriers.  tab: the
+// ColTw<N, VAR> table; PRUNED: the inputs of the zero band are zero; PK:
+// packed complex adds (half the issue slots; the passes that hold one line per
+// thread take them, the fused x passes have no registers to spare for the
+// pairs' alignment).
+template <int N, bool FWD, int VAR = 0, bool PRUNED = false, bool PK = false, class At, class Sync = BlockSync>
+__device__ __forceinline__ void fft_line(float2 *v, int p, const float2 *__restrict__ tab, At at, Sync sync = Sync())
 {
     using PI = PlanInfo<N, VAR>;
     constexpr int P = PI::P;
-    pass_regs<N, PI::R0, 1, P, FWD>(v, p, tw);
+    first_pass<N, FWD, VAR, PK, PRUNED>(v);
     exchange<N, PI::R0, 1, PI::R1, P>(v, p, at, sync);
-    pass_regs<N, PI::R1, PI::R0, P, FWD>(v, p, tw);
+    pass_regs_ct<N, PI::R1, PI::R0, P, FWD, PK>(v, p, tab);
     if constexpr (PI::NP == 3) {
         exchange<N, PI::R1, PI::R0, PI::R2, P>(v, p, at, sync);
-        pass_regs<N, PI::R2, PI::R0 * PI::R1, P, FWD>(v, p, tw);
+        pass_regs_ct<N, PI::R2, PI::R0 * PI::R1, P, FWD, PK>(v, p, tab + ColTw<N, VAR>::OFF2);
     }
 }
 
@@ -386,7 +540,29 @@ struct WPlanInfo {
     static_assert(V % R0 == 0 && V % R1 == 0 && V % R2 == 0 && V % R3 == 0, "radix must divide V");
     static __device__ __forceinline__ int in_pos(int p, int i) { return p + (i / R0) * P + (i % R0) * (N / R0); }
     static __device__ __forceinline__ int out_pos(int p, int i) { return p + (i / RL) * P + (i % RL) * (N / RL); }
+    // first-pass inputs of butterfly b of a Hermitian line that lie in the zero band for every lane
+    static __host__ __device__ constexpr unsigned zeros(int b)
+    {
+        const int KC = (N + 2) / 3 - 1;
+        unsigned m = 0;
+        for (int t = 0; t < R0; ++t) {
+            const int c = b * P + t * (N / R0);
+            if (c > KC && c + P - 1 < N - KC) m |= 1u << t;
+        }
+        return m;
+    }
 };
+
+// first pass of a warp-local line; PRUNED: the zero band's inputs are zero
+template <int N, int VAR, bool FWD, bool PRUNED, int B = 0>
+__device__ __forceinline__ void first_pass_warp(float2 *v)
+{
+    using PI = WPlanInfo<N, VAR>;
+    if constexpr (B < PI::V / PI::R0) {
+        Dft<PI::R0, FWD, true, PRUNED ? PI::zeros(B) : 0u>::run(&v[B * PI::R0]);
+        first_pass_warp<N, VAR, FWD, PRUNED, B + 1>(v);
+    }
+}
 
 template <int N, int R, int Ns, int Rn, int P, class At>
 __device__ __forceinline__ void exchange_warp(float2 *v, int p, At at)
@@ -567,7 +743,7 @@ __device__ __forceinline__ void pass_regs_lt(float2 *v, const float2 *__restrict
 
 // Line transform of the default warp plan through the padded layouts with
 // the lane-major shared twiddles (tab: LaneTw<N> table).
-template <int N, bool FWD>
+template <int N, bool FWD, bool PRUNED = false>
 __device__ __forceinline__ void fft_line_warp_pad_lt(float2 *v, int p, const float2 *__restrict__ tab, float2 *row)
 {
     using PI = WPlanInfo<N, 0>;
@@ -575,7 +751,7 @@ __device__ __forceinline__ void fft_line_warp_pad_lt(float2 *v, int p, const flo
     using LT = LaneTw<N>;
     static_assert(PD::on && PI::NP <= 3, "padded layouts exist for the power-of-two plans");
     constexpr int P = PI::P, R0 = PI::R0, R1 = PI::R1, R2 = PI::R2;
-    pass_regs<N, R0, 1, P, FWD, true>(v, p, nullptr);
+    first_pass_warp<N, 0, FWD, PRUNED>(v);
     exchange_warp_pad<N, R0, 1, R1, P, PD::A0, PD::D0>(v, p, row);
     pass_regs_lt<N, R1, R0, P, FWD, true>(v, tab + p);
     if constexpr (PI::NP == 3) {
@@ -586,14 +762,14 @@ __device__ __forceinline__ void fft_line_warp_pad_lt(float2 *v, int p, const flo
 
 // Line transform of a warp plan through the padded layouts; row is this
 // line's shared row (WPadV<N, VAR>::SROW slots).
-template <int N, bool FWD, int VAR = 0>
+template <int N, bool FWD, int VAR = 0, bool PRUNED = false>
 __device__ __forceinline__ void fft_line_warp_pad(float2 *v, int p, const WarpTw<N, VAR> &T, float2 *row)
 {
     using PI = WPlanInfo<N, VAR>;
     using PD = WPadV<N, VAR>;
     static_assert(PD::on && PI::NP <= 3, "padded layouts exist for the power-of-two plans");
     constexpr int P = PI::P, R0 = PI::R0, R1 = PI::R1, R2 = PI::R2;
-    pass_regs<N, R0, 1, P, FWD, true>(v, p, nullptr);
+    first_pass_warp<N, VAR, FWD, PRUNED>(v);
     exchange_warp_pad<N, R0, 1, R1, P, PD::A0, PD::D0>(v, p, row);
     pass_regs_tw<N, R1, R0, P, FWD, true>(v, T.t1);
     if constexpr (PI::NP == 3) {
@@ -603,13 +779,13 @@ __device__ __forceinline__ void fft_line_warp_pad(float2 *v, int p, const WarpTw
 }
 
 // Warp-local line transform with register twiddles.
-template <int N, bool FWD, int VAR = 0, class At>
+template <int N, bool FWD, int VAR = 0, bool PRUNED = false, class At>
 __device__ __forceinline__ void fft_line_warp_tw(float2 *v, int p, const WarpTw<N, VAR> &T, At at)
 {
     using PI = WPlanInfo<N, VAR>;
     constexpr int P = PI::P;
     constexpr int R0 = PI::R0, R1 = PI::R1, R2 = PI::R2, R3 = PI::R3;
-    pass_regs<N, R0, 1, P, FWD, true>(v, p, nullptr);
+    first_pass_warp<N, VAR, FWD, PRUNED>(v);
     exchange_warp<N, R0, 1, R1, P>(v, p, at);
     pass_regs_tw<N, R1, R0, P, FWD, true>(v, T.t1);
     if constexpr (PI::NP >= 3) {
@@ -623,13 +799,13 @@ __device__ __forceinline__ void fft_line_warp_tw(float2 *v, int p, const WarpTw<
 }
 
 // Warp-local line transform; all 32 lanes of the warp must call it.
-template <int N, bool FWD, class At>
+template <int N, bool FWD, bool PRUNED = false, class At>
 __device__ __forceinline__ void fft_line_warp(float2 *v, int p, const float2 *__restrict__ tw, At at)
 {
     using PI = WPlanInfo<N>;
     constexpr int P = PI::P;
     constexpr int R0 = PI::R0, R1 = PI::R1, R2 = PI::R2, R3 = PI::R3;
-    pass_regs<N, R0, 1, P, FWD, true>(v, p, tw);
+    first_pass_warp<N, 0, FWD, PRUNED>(v);
     exchange_warp<N, R0, 1, R1, P>(v, p, at);
     pass_regs<N, R1, R0, P, FWD, true>(v, p, tw);
     if constexpr (PI::NP >= 3) {

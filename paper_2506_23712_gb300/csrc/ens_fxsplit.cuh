@@ -29,30 +29,26 @@ template <int N, int T>
 __global__ void __launch_bounds__(ColCfg<N, T>::threads)
 k_fwd_x_fft(Geo g)
 {
-    using PI = PlanInfo<N>;
-    constexpr int P = PI::P, V = PI::V;
+    constexpr int V = PlanInfo<N>::V;
     extern __shared__ __align__(16) float2 sm[];
+    using CS = ColSlots<N, 0>;
     float2 *tw = sm, *buf = sm + N;
-    load_twiddles(tw, g.tw, N);
+    load_col_twiddles<N, 0>(tw, g.tw);
     const int c = threadIdx.x % T, p = threadIdx.x / T;
     const int q = blockIdx.y, m = blockIdx.z;
     const int col = blockIdx.x * T + c;                  // (ky, kz) flat
     const int iy = col / Dims<N>::NZP, kz = col % Dims<N>::NZP;
     const bool valid = kz < Dims<N>::NZ;
-    const float2 *src = g.A + ((long long)m * kFields + q) * Dims<N>::SA + ((long long)iy * N) * Dims<N>::NZP + kz;
-    float2 *dst = nhat_of<N>(g, m) + q * Dims<N>::SU + col;
-    constexpr long long rowU = (long long)Dims<N>::NK * Dims<N>::NZP;
+    const float2 *src = g.A + ((long long)m * kFields + q) * Dims<N>::SA + ((long long)iy * N + p) * Dims<N>::NZP + kz;
+    constexpr unsigned rowU = Dims<N>::NK * Dims<N>::NZP;
+    float2 *dst = nhat_of<N>(g, m) + q * Dims<N>::SU;
+    const unsigned off = p * rowU + col;
     float2 v[V];
 #pragma unroll
-    for (int i = 0; i < V; ++i) v[i] = valid ? src[(long long)PI::in_pos(p, i) * Dims<N>::NZP] : make_float2(0.f, 0.f);
-    fft_line<N, true>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
-    if (valid) {
-#pragma unroll
-        for (int i = 0; i < V; ++i) {
-            const int kx = wnum(PI::out_pos(p, i), N);
-            if (kx >= -Dims<N>::KC && kx <= Dims<N>::KC) dst[(kx >= 0 ? kx : kx + Dims<N>::NK) * rowU] = v[i];
-        }
-    }
+    for (int i = 0; i < V; ++i) v[i] = valid ? src[CS::in(i) * Dims<N>::NZP] : make_float2(0.f, 0.f);
+    fft_line<N, true, 0, false, true>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
+    store_kept<N, 0>(v, p, kz < Dims<N>::NZS,
+                     [&](auto s, float2 w) { at32(dst, off + (unsigned)CS::row(s.value) * rowU) = w; });
 }
 
 constexpr int kUpdThreads = 256;
@@ -112,8 +108,8 @@ __device__ __forceinline__ float update_mode(const UpdCoef &c, int kx, int ky, i
 // grid (update_blocks<N>(), members), block kUpdThreads.  Thread t takes
 // the mode pairs (2j, 2j + 1), j = first + t + u * kUpdThreads: 16-byte
 // loads and stores, and every load of a pair issued before its arithmetic.
-// A pair never straddles a kz row (NZp is even); a mode past the kept kz
-// (odd NZ) is written as zero, a pair wholly past it is not touched.
+// A pair never straddles a kz row (NZp is even); modes past the kept kz are
+// written as zero up to the end of their 64 bytes.
 template <int N>
 __global__ void __launch_bounds__(kUpdThreads, 4)
 k_update(Geo g, MemberDev *md, int stage, int last_stage)
@@ -150,15 +146,15 @@ k_update(Geo g, MemberDev *md, int stage, int last_stage)
         const int ix = (int)(mi / rowU);
         const int rem = (int)(mi % rowU);
         const int iy = rem / D::NZP, kz = rem % D::NZP;
-        const bool any = j < SU2 && kz < D::NZ;
-        const bool both = any && kz + 1 < D::NZ;
+        const bool any = j < SU2 && kz < D::NZS;
         float4 n4[3], u4[3], s4[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            n4[q] = any ? nh[q * SU2 + j] : z4;
-            u4[q] = any ? U[q * SU2 + j] : z4;
-            s4[q] = (any && stage != 0) ? S[q * SU2 + j] : u4[q];
+            const bool ld = any && kz < D::NZ;
+            n4[q] = ld ? nh[q * SU2 + j] : z4;
+            u4[q] = ld ? U[q * SU2 + j] : z4;
+            s4[q] = (ld && stage != 0) ? S[q * SU2 + j] : u4[q];
         }
         if (!any) continue;
         const int kx = ix <= D::KC ? ix : ix - D::NK;
@@ -176,7 +172,7 @@ k_update(Geo g, MemberDev *md, int stage, int last_stage)
             bool band;
             float k2;
             const float a2 = update_mode(c, kx, ky, kz + h, n, un, us, o, band, k2);
-            const bool keep = h == 0 || both;
+            const bool keep = kz + h < D::NZ;
             const float wgt = (kz + h) == 0 ? 1.f : 2.f;   // Hermitian multiplicity in the full spectrum
             if (keep) {
                 se += 0.5f * wgt * a2;

@@ -55,8 +55,7 @@ k_fwd_x_ws(Geo g, MemberDev *md, int stage, int last_stage)
     extern __shared__ __align__(16) float2 sm[];
     __shared__ double red[(TH / 32) * 3];
     float2 *tw = sm, *buf = sm + N, *tiles = buf + N * T;   // tiles: [2][3][NK][T]
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = g.tw[i];
-    __syncthreads();
+    load_col_twiddles<N, 0>(tw, g.tw);
     const long long ntiles = (long long)C::TILES * g.members;
     const int nk = ntiles > blockIdx.x ? (int)((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;   // tiles of this CTA
     const int lt = threadIdx.x % TH;
@@ -86,12 +85,9 @@ k_fwd_x_ws(Geo g, MemberDev *md, int stage, int last_stage)
                                        : make_float2(0.f, 0.f);
                 }
                 fft_line<N, true, 0>(v, p, tw, at, NamedSync<5, TH>());
-#pragma unroll
-                for (int i = 0; i < V; ++i) {
-                    const int kx = wnum(PI::out_pos(p, i), N);
-                    if (kx >= -Dims<N>::KC && kx <= Dims<N>::KC)
-                        tile[q * PER + (kx >= 0 ? kx : kx + Dims<N>::NK) * T + c] = v[i];
-                }
+                float2 *dt = tile + q * PER + p * T + c;
+                store_kept<N, 0>(v, p, true,
+                                 [&](auto s, float2 w) { dt[ColSlots<N, 0>::row(s.value) * T] = w; });
                 if (q < 2) {
 #pragma unroll
                     for (int i = 0; i < V; ++i) v[i] = nxt[i];
@@ -148,7 +144,8 @@ k_fwd_x_ws(Geo g, MemberDev *md, int stage, int last_stage)
                     if (idx >= PER) continue;
                     const int ix = idx / T, cc = idx % T;
                     const int kzc = kz0 + cc;
-                    if (kzc >= Dims<N>::NZ) continue;
+                    if (kzc >= Dims<N>::NZS) continue;   // zeros to the end of the row's 64 bytes
+                    const bool keep = kzc < Dims<N>::NZ;
                     const int kx = ix <= Dims<N>::KC ? ix : ix - Dims<N>::NK;
                     const float fk[3] = {(float)kx, (float)kyi, (float)kzc};
                     const int k2i = kx * kx + kyi * kyi + kzc * kzc;
@@ -184,9 +181,10 @@ k_fwd_x_ws(Geo g, MemberDev *md, int stage, int last_stage)
                         const float rx = us[q].x + dtf * n[q].x, ry = us[q].y + dtf * n[q].y;
                         const float ox = if_combine(ic, un[q].x, rx);
                         const float oy = if_combine(ic, un[q].y, ry);
-                        dst[q * Dims<N>::SU + off] = make_float2(ox, oy);
+                        dst[q * Dims<N>::SU + off] = keep ? make_float2(ox, oy) : make_float2(0.f, 0.f);
                         a2 += ox * ox + oy * oy;
                     }
+                    if (!keep) a2 = 0.f;
                     se += 0.5f * wgt * a2;
                     sd += nu * k2 * wgt * a2;
                     if (band) sb += 0.5f * wgt * a2;

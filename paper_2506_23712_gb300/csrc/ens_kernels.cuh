@@ -34,6 +34,11 @@ struct Dims {
     static constexpr int NK = 2 * KC + 1;
     static constexpr int NZ = KC + 1;
     static constexpr int NZP = (NZ + kTile - 1) / kTile * kTile;
+    // columns written per row: NZ rounded up to 64 bytes, zeros past NZ.  A row
+    // that ends inside a 32-byte sector makes the memory read the rest of the
+    // last burst before it can be written back: 64 bytes read per row written
+    // (256^3 y pass: 855 MB read for 723 MB of input; 64^3: 317 for 186).
+    static constexpr int NZS = (NZ + 7) / 8 * 8;
     static constexpr long long SU = (long long)NK * NK * NZP;   // per state component
     static constexpr long long SA = (long long)NK * N * NZP;    // per buffer-A field
     static constexpr long long SB = (long long)N * N * NZP;     // per buffer-B field
@@ -90,8 +95,6 @@ constexpr size_t smem_x() { return smem_cols<N, T>() + sizeof(float2) * 3 * (2 *
 template <int N>
 constexpr size_t smem_rows() { return sizeof(float2) * (size_t)(N + RowCfg<N>::RZ * RowCfg<N>::SROW); }
 
-__device__ __forceinline__ int wnum(int pos, int N) { return pos <= N / 2 ? pos : pos - N; }
-
 // 16-byte asynchronous global -> shared copy (cp.async, L2 only); bytes < 16
 // of the source are read and the rest of the destination is zero-filled
 __device__ __forceinline__ void cp_async_16(void *dst, const void *src, int bytes)
@@ -121,6 +124,18 @@ __device__ __forceinline__ void load_twiddles(float2 *tw, const float2 *__restri
     __syncthreads();
 }
 
+// the inter-pass twiddles of a column plan, whole block
+template <int N, int VAR>
+__device__ __forceinline__ void load_col_twiddles(float2 *tab, const float2 *__restrict__ g)
+{
+    ColTw<N, VAR>::load(tab, g, threadIdx.x, blockDim.x);
+    __syncthreads();
+}
+
+// element `off` (32-bit, from a base that is the same for the whole block)
+__device__ __forceinline__ const float2 &at32(const float2 *base, unsigned off) { return base[off]; }
+__device__ __forceinline__ float2 &at32(float2 *base, unsigned off) { return base[off]; }
+
 // ---------------------------------------------------------------------------
 // IX: inverse transform along x of fields built from the state.
 //   MODE 0: u_x, u_y, u_z, omega_x, omega_y, omega_z   (omega = i k x u)
@@ -143,7 +158,7 @@ __device__ __forceinline__ void inv_x_body(const Geo &g, int use_S, int bx, int 
     const int col = col0 + c;
     const int iy = col / Dims<N>::NZP, kz = col % Dims<N>::NZP;
     const int kz0 = col0 % Dims<N>::NZP;                  // first kz of the tile
-    const bool valid = kz < Dims<N>::NZ;
+    const bool stored = kz < Dims<N>::NZS;
     const float ky = (float)(iy <= Dims<N>::KC ? iy : iy - Dims<N>::NK);
     const float kzf = (float)kz;
     const long long rowU = (long long)Dims<N>::NK * Dims<N>::NZP;
@@ -165,7 +180,7 @@ __device__ __forceinline__ void inv_x_body(const Geo &g, int use_S, int bx, int 
         }
         cp_async_commit();
     }
-    load_twiddles(tw, g.tw, N);
+    load_col_twiddles<N, VAR>(tw, g.tw);
     // component order[s] complete and visible to the block
     auto landed = [&](int s) {
         if (s == 0) cp_async_wait<2>();
@@ -179,18 +194,30 @@ __device__ __forceinline__ void inv_x_body(const Geo &g, int use_S, int bx, int 
     // transform of component q of the tile, optionally times i kx (the x
     // derivative: kx varies along this transform, so it is applied before it)
     auto transform = [&](float2 *v, int q, bool dx) {
+        using CS = ColSlots<N, VAR>;
+        const float2 *src = tile + q * per + p * T + c;
+        if constexpr (MODE == 0) {
+            load_kept<N, VAR>(v, p, true, [&](auto s) {
+                const float2 u = src[CS::row(s.value) * T];
+                return dx ? mul_i(cscale(u, (float)(p + CS::wave(s.value)))) : u;
+            });
+            fft_line<N, false, VAR, true>(v, p, tw, at);
+        } else {
+            // statistics: every slot is multiplied and every butterfly formed, so
+            // that the products by kx round as they always have (contracted into
+            // the first additions) and the histogram counts stay the same
+            load_kept<N, VAR>(v, p, true, [&](auto s) { return src[CS::row(s.value) * T]; });
+            if (dx) {
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            const int kxi = wnum(PI::in_pos(p, i), N);
-            const bool keep = kxi >= -Dims<N>::KC && kxi <= Dims<N>::KC;
-            const int ix = kxi >= 0 ? kxi : kxi + Dims<N>::NK;
-            const float2 u = keep ? tile[q * per + ix * T + c] : make_float2(0.f, 0.f);
-            v[i] = dx ? mul_i(cscale(u, (float)kxi)) : u;
+                for (int i = 0; i < V; ++i) v[i] = mul_i(cscale(v[i], (float)(p + CS::wave(CS::in(i)))));
+                fft_line<N, false, VAR, false>(v, p, tw, at);
+            } else {
+                fft_line<N, false, VAR, true>(v, p, tw, at);
+            }
         }
-        fft_line<N, false, VAR>(v, p, tw, at);
     };
     auto store = [&](const float2 *v, int f) {
-        if (valid) {
+        if (stored) {
             float2 *dst = dst0 + (long long)f * Dims<N>::SA;
 #pragma unroll
             for (int i = 0; i < V; ++i) dst[(long long)PI::out_pos(p, i) * Dims<N>::NZP] = v[i];
@@ -257,26 +284,22 @@ __device__ __forceinline__ void inv_y_body(const Geo &g, int bx, int f, int m, f
 {
     using PI = PlanInfo<N, VAR>;
     constexpr int P = PI::P, V = PI::V;
+    using CS = ColSlots<N, VAR>;
     float2 *tw = sm, *buf = sm + N;
-    load_twiddles(tw, g.tw, N);
+    load_col_twiddles<N, VAR>(tw, g.tw);
     const int c = threadIdx.x % T, p = threadIdx.x / T;
     const int col = bx * T + c;               // (x, kz) flat
-    const bool valid = (col % Dims<N>::NZP) < Dims<N>::NZ;
-    const long long row = (long long)N * Dims<N>::NZP;
-    const float2 *src = g.A + ((long long)m * kFields + f) * Dims<N>::SA + col;
-    float2 *dst = g.B + ((long long)m * kFields + f) * Dims<N>::SB + col;
+    const bool valid = (col % Dims<N>::NZP) < Dims<N>::NZ, stored = (col % Dims<N>::NZP) < Dims<N>::NZS;
+    constexpr unsigned row = N * Dims<N>::NZP;
+    const float2 *src = g.A + ((long long)m * kFields + f) * Dims<N>::SA;
+    float2 *dst = g.B + ((long long)m * kFields + f) * Dims<N>::SB;
+    const unsigned off = p * row + col;
     float2 v[V];
+    load_kept<N, VAR>(v, p, valid, [&](auto s) { return at32(src, off + (unsigned)CS::row(s.value) * row); });
+    fft_line<N, false, VAR, true, true>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
+    if (stored) {
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const int ky = wnum(PI::in_pos(p, i), N);
-        const bool keep = valid && ky >= -Dims<N>::KC && ky <= Dims<N>::KC;
-        const int iy = ky >= 0 ? ky : ky + Dims<N>::NK;
-        v[i] = keep ? src[iy * row] : make_float2(0.f, 0.f);
-    }
-    fft_line<N, false, VAR>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
-    if (valid) {
-#pragma unroll
-        for (int i = 0; i < V; ++i) dst[PI::out_pos(p, i) * row] = v[i];
+        for (int i = 0; i < V; ++i) at32(dst, off + (unsigned)CS::out(i) * row) = v[i];
     }
 }
 
@@ -312,7 +335,8 @@ k_inv_y_grad(Geo g)
     constexpr int P = PI::P, V = PI::V;
     extern __shared__ __align__(16) float2 sm[];
     float2 *tw = sm, *buf = sm + N;
-    load_twiddles(tw, g.tw, N);
+    load_col_twiddles<N, 0>(tw, g.tw);
+    using CS = ColSlots<N, 0>;
     const int fo = blockIdx.x, m = blockIdx.z;
     const int ci = fo / 3, jj = fo % 3;
     const int fi = jj == 0 ? 3 + ci : ci;
@@ -320,27 +344,23 @@ k_inv_y_grad(Geo g)
     const int col = blockIdx.y * T + c;        // (x, kz) flat
     const int kz = col % Dims<N>::NZP;
     const bool valid = kz < Dims<N>::NZ;
-    const long long row = (long long)N * Dims<N>::NZP;
-    const float2 *src = g.A + ((long long)m * kFields + fi) * Dims<N>::SA + col;
+    constexpr unsigned row = N * Dims<N>::NZP;
+    const float2 *src = g.A + ((long long)m * kFields + fi) * Dims<N>::SA;
+    const unsigned off = p * row + col;
     float2 v[V];
+    load_kept<N, 0>(v, p, valid, [&](auto s) { return at32(src, off + (unsigned)CS::row(s.value) * row); });
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const int ky = wnum(PI::in_pos(p, i), N);
-        const bool keep = valid && ky >= -Dims<N>::KC && ky <= Dims<N>::KC;
-        const int iy = ky >= 0 ? ky : ky + Dims<N>::NK;
-        const float2 u = keep ? src[iy * row] : make_float2(0.f, 0.f);
-        v[i] = jj == 1 ? mul_i(cscale(u, (float)ky)) : u;
-    }
-    fft_line<N, false, 0>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
+    for (int i = 0; i < V; ++i) v[i] = jj == 1 ? mul_i(cscale(v[i], (float)(p + CS::wave(CS::in(i))))) : v[i];
+    fft_line<N, false, 0, true, true>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
     if (jj == 2) {
         const float kzf = (float)kz;
 #pragma unroll
         for (int i = 0; i < V; ++i) v[i] = mul_i(cscale(v[i], kzf));
     }
-    if (valid) {
-        float2 *dst = g.B + ((long long)m * kFields + fo) * Dims<N>::SB + col;
+    if (kz < Dims<N>::NZS) {
+        float2 *dst = g.B + ((long long)m * kFields + fo) * Dims<N>::SB;
 #pragma unroll
-        for (int i = 0; i < V; ++i) dst[PI::out_pos(p, i) * row] = v[i];
+        for (int i = 0; i < V; ++i) at32(dst, off + (unsigned)CS::out(i) * row) = v[i];
     }
 }
 
@@ -353,25 +373,22 @@ __device__ __forceinline__ void fwd_y_body(const Geo &g, int bx, int f, int m, f
 {
     using PI = PlanInfo<N, VAR>;
     constexpr int P = PI::P, V = PI::V;
+    using CS = ColSlots<N, VAR>;
     float2 *tw = sm, *buf = sm + N;
-    load_twiddles(tw, g.tw, N);
+    load_col_twiddles<N, VAR>(tw, g.tw);
     const int c = threadIdx.x % T, p = threadIdx.x / T;
     const int col = bx * T + c;
-    const bool valid = (col % Dims<N>::NZP) < Dims<N>::NZ;
-    const long long row = (long long)N * Dims<N>::NZP;
-    const float2 *src = g.B + ((long long)m * kFields + f) * Dims<N>::SB + col;
-    float2 *dst = g.A + ((long long)m * kFields + f) * Dims<N>::SA + col;
+    const bool valid = (col % Dims<N>::NZP) < Dims<N>::NZ, stored = (col % Dims<N>::NZP) < Dims<N>::NZS;
+    constexpr unsigned row = N * Dims<N>::NZP;
+    const float2 *src = g.B + ((long long)m * kFields + f) * Dims<N>::SB;
+    float2 *dst = g.A + ((long long)m * kFields + f) * Dims<N>::SA;
+    const unsigned off = p * row + col;
     float2 v[V];
 #pragma unroll
-    for (int i = 0; i < V; ++i) v[i] = valid ? src[PI::in_pos(p, i) * row] : make_float2(0.f, 0.f);
-    fft_line<N, true, VAR>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
-    if (valid) {
-#pragma unroll
-        for (int i = 0; i < V; ++i) {
-            const int ky = wnum(PI::out_pos(p, i), N);
-            if (ky >= -Dims<N>::KC && ky <= Dims<N>::KC) dst[(ky >= 0 ? ky : ky + Dims<N>::NK) * row] = v[i];
-        }
-    }
+    for (int i = 0; i < V; ++i) v[i] = valid ? at32(src, off + (unsigned)CS::in(i) * row) : make_float2(0.f, 0.f);
+    fft_line<N, true, VAR, false, true>(v, p, tw, [&](int pos) { return &buf[pos * T + c]; });
+    store_kept<N, VAR>(v, p, stored,
+                       [&](auto s, float2 w) { at32(dst, off + (unsigned)CS::row(s.value) * row) = w; });
 }
 
 template <int N, int T, int VAR = 0>
@@ -711,8 +728,9 @@ __device__ __forceinline__ void fwd_x_body(const Geo &g, MemberDev *md, int stag
 {
     using PI = PlanInfo<N, VAR>;
     constexpr int P = PI::P, V = PI::V;
+    using CS = ColSlots<N, VAR>;
     float2 *tw = sm, *buf = sm + N, *tile = buf + N * T;   // tile: [3][NK][T]
-    load_twiddles(tw, g.tw, N);
+    load_col_twiddles<N, VAR>(tw, g.tw);
     const int c = threadIdx.x % T, p = threadIdx.x / T;
     const int col0 = bx * T;
     const int col = col0 + c;                                  // (ky, kz) flat
@@ -737,11 +755,8 @@ __device__ __forceinline__ void fwd_x_body(const Geo &g, MemberDev *md, int stag
                                : make_float2(0.f, 0.f);
         }
         fft_line<N, true, VAR>(v, p, tw, at);
-#pragma unroll
-        for (int i = 0; i < V; ++i) {
-            const int kx = wnum(PI::out_pos(p, i), N);
-            if (kx >= -Dims<N>::KC && kx <= Dims<N>::KC) tile[q * per + (kx >= 0 ? kx : kx + Dims<N>::NK) * T + c] = v[i];
-        }
+        float2 *dt = tile + q * per + p * T + c;
+        store_kept<N, VAR>(v, p, true, [&](auto s, float2 w) { dt[CS::row(s.value) * T] = w; });
         if (q < 2) {
 #pragma unroll
             for (int i = 0; i < V; ++i) v[i] = nxt[i];
@@ -795,7 +810,9 @@ __device__ __forceinline__ void fwd_x_body(const Geo &g, MemberDev *md, int stag
         if (idx >= per) continue;
         const int ix = idx / T, cc = idx % T;
         const int kzc = kz0 + cc;
-        if (kzc >= Dims<N>::NZ) continue;
+        // columns past the kept modes: zeros to the end of the row's 64 bytes
+        if (kzc >= (MODE == 0 || MODE == 1 ? Dims<N>::NZS : Dims<N>::NZ)) continue;
+        const bool keep = kzc < Dims<N>::NZ;
         const int kx = ix <= Dims<N>::KC ? ix : ix - Dims<N>::NK;
         const float fk[3] = {(float)kx, (float)kyi, (float)kzc};
         const int k2i = kx * kx + kyi * kyi + kzc * kzc;
@@ -838,7 +855,7 @@ __device__ __forceinline__ void fwd_x_body(const Geo &g, MemberDev *md, int stag
             }
             if constexpr (MODE == 1) {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) S[q * Dims<N>::SU + off] = n[q];
+                for (int q = 0; q < 3; ++q) S[q * Dims<N>::SU + off] = keep ? n[q] : make_float2(0.f, 0.f);
             } else {
                 const IfCoef ic = if_coef(co, nu, k2, dtf);
                 float2 *dst = last_stage ? U : S;
@@ -848,9 +865,10 @@ __device__ __forceinline__ void fwd_x_body(const Geo &g, MemberDev *md, int stag
                     const float rx = us[q].x + dtf * n[q].x, ry = us[q].y + dtf * n[q].y;
                     const float ox = if_combine(ic, un[q].x, rx);
                     const float oy = if_combine(ic, un[q].y, ry);
-                    dst[q * Dims<N>::SU + off] = make_float2(ox, oy);
+                    dst[q * Dims<N>::SU + off] = keep ? make_float2(ox, oy) : make_float2(0.f, 0.f);
                     a2 += ox * ox + oy * oy;
                 }
+                if (!keep) a2 = 0.f;
                 se += 0.5f * wgt * a2;
                 sd += nu * k2 * wgt * a2;
                 if (band) sb += 0.5f * wgt * a2;

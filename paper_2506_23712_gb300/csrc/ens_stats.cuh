@@ -264,8 +264,8 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            if constexpr (C::PAD) fft_line_warp_pad_lt<N, false>(v[q], p, ltw, myrow);
-            else fft_line_warp<N, false>(v[q], p, tw, at);
+            if constexpr (C::PAD) fft_line_warp_pad_lt<N, false, true>(v[q], p, ltw, myrow);
+            else fft_line_warp<N, false, true>(v[q], p, tw, at);
         }
 #pragma unroll
         for (int i = 0; i < V; ++i) {

@@ -161,6 +161,7 @@ __device__ __forceinline__ void forward_pair_store_shfl(float2 *v, int p, int li
     constexpr int P = PI::P, V = PI::V, NZ = Dims<N>::NZ;
     static_assert(PI::RL == V, "the last pass must hold one butterfly per lane");
     static_assert((NZ + P - 1) / P <= V, "unpacking rounds exceed the slots");
+    static_assert((NZ + P - 1) / P * P >= Dims<N>::NZS, "unpacking rounds end before the written columns");
     fft_line_warp_pad<N, true, VAR>(v, p, T, row);
     const int src = line * P + ((P - p) & (P - 1));
 #pragma unroll
@@ -169,12 +170,13 @@ __device__ __forceinline__ void forward_pair_store_shfl(float2 *v, int p, int li
         const float2 z = v[i];
         const float2 w = make_float2(__shfl_sync(0xffffffffu, send.x, src), -__shfl_sync(0xffffffffu, send.y, src));
         const int k = p + i * P;
-        if (k < NZ) {
-            // Xa = (Z_k + conj Z_{N-k}) / 2 ; Xb = (Z_k - conj Z_{N-k}) / (2i)
-            dstA[k] = cscale_x2(0.5f, cadd_x2(z, w));
+        if (k < Dims<N>::NZS) {
+            // Xa = (Z_k + conj Z_{N-k}) / 2 ; Xb = (Z_k - conj Z_{N-k}) / (2i); zeros past the kept modes
+            const bool keep = k < NZ;
+            dstA[k] = keep ? cscale_x2(0.5f, cadd_x2(z, w)) : make_float2(0.f, 0.f);
             if (dstB) {
                 const float2 d = csub_x2(z, w);
-                dstB[k] = make_float2(0.5f * d.y, -0.5f * d.x);
+                dstB[k] = keep ? make_float2(0.5f * d.y, -0.5f * d.x) : make_float2(0.f, 0.f);
             }
         }
     }
@@ -284,13 +286,13 @@ __device__ __forceinline__ void znl_body(const Geo &g, MemberDev *md, int stage_
         PairSlots<N, VAR, 0>::load(bb, X + 2 * R, X + 3 * R, p);
         PairSlots<N, VAR, 0>::load(cc, X + 4 * R, X + 5 * R, p);
         if constexpr (C::PAD) {
-            fft_line_warp_pad<N, false, VAR>(a, p, TW, myrow);
-            fft_line_warp_pad<N, false, VAR>(bb, p, TW, myrow);
-            fft_line_warp_pad<N, false, VAR>(cc, p, TW, myrow);
+            fft_line_warp_pad<N, false, VAR, true>(a, p, TW, myrow);
+            fft_line_warp_pad<N, false, VAR, true>(bb, p, TW, myrow);
+            fft_line_warp_pad<N, false, VAR, true>(cc, p, TW, myrow);
         } else {
-            fft_line_warp_tw<N, false, VAR>(a, p, TW, at);
-            fft_line_warp_tw<N, false, VAR>(bb, p, TW, at);
-            fft_line_warp_tw<N, false, VAR>(cc, p, TW, at);
+            fft_line_warp_tw<N, false, VAR, true>(a, p, TW, at);
+            fft_line_warp_tw<N, false, VAR, true>(bb, p, TW, at);
+            fft_line_warp_tw<N, false, VAR, true>(cc, p, TW, at);
         }
         // a = ux + i uy, bb = uz + i wx, cc = wy + i wz at positions out_pos;
         // the CFL step takes max|u_i| of the first stage only

@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -1035,6 +1036,43 @@ ens_status ens_mixture(ens_ctx *ctx, const ens_weight_spec *w, ens_mixture_out *
     return ENS_OK;
 }
 
+// Device scratch of ens_mixture_host: a memory pool of the library's own per
+// device, which keeps at most kScratchKeep bytes between calls (more goes back
+// to the device at the next synchronisation), so that repeated calls do not
+// map and unmap their few megabytes each time (170 us a call with the default
+// pool, which keeps nothing; a pool maps 32 MB at a time, and keeps nothing
+// either where it may keep less than that).  Stream-ordered, safe with several
+// threads and streams; the default pool where the device has no pools.
+static cudaError_t scratch_alloc(void **mem, size_t bytes, cudaStream_t st)
+{
+    constexpr int kMaxDev = 64;
+    constexpr unsigned long long kScratchKeep = 32ull << 20;
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxDev] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    if (dev < kMaxDev) {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps pr{};
+            pr.allocType = cudaMemAllocationTypePinned;
+            pr.location.type = cudaMemLocationTypeDevice;
+            pr.location.id = dev;
+            unsigned long long keep = kScratchKeep;
+            if (cudaMemPoolCreate(&pools[dev], &pr) != cudaSuccess) {
+                pools[dev] = nullptr;
+                cudaGetLastError();
+            } else {
+                cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+            }
+        }
+        pool = pools[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(mem, bytes, pool, st) : cudaMallocAsync(mem, bytes, st);
+}
+
 ens_status ens_mixture_host(int n, const double *lambdas, const uint64_t *counts, const double *moments,
                             const ens_hist_spec *h, const ens_weight_spec *w, ens_mixture_out *out, void *stream)
 {
@@ -1047,7 +1085,7 @@ ens_status ens_mixture_host(int n, const double *lambdas, const uint64_t *counts
     const size_t nd = (size_t)3 * n + 1 + L + kNMom + 8 + (size_t)n * kNMom;
     const size_t bytes = sizeof(double) * nd + sizeof(unsigned long long) * n * L;
     void *mem = nullptr;
-    if (cudaMallocAsync(&mem, bytes, st) != cudaSuccess) return ENS_ENOMEM;
+    if (scratch_alloc(&mem, bytes, st) != cudaSuccess) return ENS_ENOMEM;
     double *d = (double *)mem;
     double *d_lam = d, *d_user = d + n, *d_mom = d + 2 * n, *d_scr = d_mom + (size_t)n * kNMom;
     unsigned long long *d_counts = reinterpret_cast<unsigned long long *>(d + nd);

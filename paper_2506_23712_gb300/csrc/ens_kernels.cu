@@ -156,16 +156,33 @@ __device__ double trunc_mu(double c, double Z)
     return 0.5 * (lo + hi);
 }
 
+// sum of one value per thread over the block (at most 1024 threads, whole
+// warps), for every thread
+__device__ double block_total(double v, double *scratch)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0.0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) v += scratch[k];
+    return v;
+}
+
+// one block, a thread per member (whole warps)
 __global__ void k_mix_weights(const double *lam, int n, MixWeightArgs wa, double *w, double *covered)
 {
     const int i = threadIdx.x;
-    __shared__ double wsh[1024];
+    __shared__ double lsh[1024], scratch[32];
+    if (i < n) lsh[i] = lam[i];
+    __syncthreads();
+    double v = 0.0;
     if (i < n) {
-        const double li = lam[i];
+        const double li = lsh[i];
         double prev = -INFINITY, next = INFINITY;
         int mult = 0;
         for (int j = 0; j < n; ++j) {
-            const double lj = lam[j];
+            const double lj = lsh[j];
             if (lj == li) ++mult;
             else if (lj < li && lj > prev) prev = lj;
             else if (lj > li && lj < next) next = lj;
@@ -178,7 +195,6 @@ __global__ void k_mix_weights(const double *lam, int n, MixWeightArgs wa, double
             lo = prev == -INFINITY ? li - 0.5 * (next - li) : 0.5 * (prev + li);
             hi = next == INFINITY ? li + 0.5 * (li - prev) : 0.5 * (li + next);
         }
-        double v = 0.0;
         if (wa.kind == 2) {
             v = wa.user[i];
         } else if (wa.kind == 0 && wa.Z == 0.0) {
@@ -192,67 +208,88 @@ __global__ void k_mix_weights(const double *lam, int n, MixWeightArgs wa, double
             const double b = fmin(hi, wa.Z);
             v = b > lo ? interval_mass(lo, b, mu, sg) / norm_cdf((wa.Z - mu) / sg) / mult : 0.0;
         }
-        wsh[i] = v;
     }
-    __syncthreads();
-    __shared__ double tot;
-    if (i == 0) {
-        double s = 0.0;
-        for (int j = 0; j < n; ++j) s += wsh[j];
-        tot = s;
-        *covered = s;
-    }
-    __syncthreads();
-    if (i < n) w[i] = (wa.renormalize && tot > 0.0) ? wsh[i] / tot : wsh[i];
-}
-
-__global__ void k_mix_pdf(const unsigned long long *counts, const double *moments, const double *w, int n,
-                          MixPdfArgs a, double *pdf, double *mom_mix)
-{
-    const int L = a.counts_len;
-    const int off_c = a.nq * a.nq + 2 * a.nt;
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < mix_pdf_len(a)) {
-        // gradient bins follow the 8 counters; 3 longitudinal and 6
-        // transverse samples per grid point
-        const bool grad = b >= off_c;
-        const int src = grad ? b + 8 : b;
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) {
-            const double npts = (double)counts[(long long)i * L + off_c + 6];
-            if (npts > 0.0) s += w[i] * (double)counts[(long long)i * L + src] / npts;
-        }
-        double width = b < a.nq * a.nq ? a.dq * a.dr : a.dt;
-        if (grad) width = a.dg * (b < off_c + a.ng ? 3.0 : 6.0);
-        pdf[b] = s / width;
-    }
-    if (blockIdx.x == 0 && threadIdx.x < kNMom) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) {
-            const double npts = (double)counts[(long long)i * L + off_c + 6];
-            if (npts > 0.0) s += w[i] * moments[(long long)i * kNMom + threadIdx.x] / npts;
-        }
-        mom_mix[threadIdx.x] = s;
-    }
+    const double tot = block_total(v, scratch);
+    if (i == 0) *covered = tot;
+    if (i < n) w[i] = (wa.renormalize && tot > 0.0) ? v / tot : v;
 }
 
 // skewness / flatness / hyper-flatness of gradient components from mixed
 // moments (Sec. VII, Eq. def_skewness_flatness and the skewness prediction),
 // isotropy-averaged over the 3 longitudinal and 6 transverse components
-__global__ void k_mix_ratios(const double *mom_mix, double *ratios)
+__device__ void mix_ratios(const double *mom_mix, double *ratios)
 {
-    if (threadIdx.x != 0) return;
     const int lon[3] = {0, 4, 8}, tra[6] = {1, 2, 3, 5, 6, 7};
     double L[4] = {0, 0, 0, 0}, T[4] = {0, 0, 0, 0};
     for (int q = 0; q < 4; ++q) {
         for (int c = 0; c < 3; ++c) L[q] += mom_mix[4 * lon[c] + q] / 3.0;
         for (int c = 0; c < 6; ++c) T[q] += mom_mix[4 * tra[c] + q] / 6.0;
     }
-    ratios[0] = L[1] / pow(L[0], 1.5);
+    ratios[0] = L[1] / (L[0] * sqrt(L[0]));
     ratios[1] = L[2] / (L[0] * L[0]);
     ratios[2] = T[2] / (T[0] * T[0]);
     ratios[3] = L[3] / (L[0] * L[0] * L[0]);
     ratios[4] = T[3] / (T[0] * T[0] * T[0]);
+}
+
+// Mixed PDF, moments and moment ratios.  Block b < last: kMixBins bins, the
+// members shared out over kMixSlices threads per bin (coalesced over the
+// bins); the last block: the moments and the ratios.  Bound by the latency of
+// the counts' loads and by FP64, two lanes per SM and clock here, hence the
+// spread over all SMs and one division per member (weight / points) instead of
+// one per member and bin: 64 members x 4608 bins 184 us with a thread per bin
+// looping over the members, 18 blocks.
+constexpr int kMixBins = 32, kMixSlices = 8;
+
+__global__ void __launch_bounds__(kMixBins * kMixSlices)
+k_mix_pdf(const unsigned long long *__restrict__ counts, const double *__restrict__ moments,
+          const double *__restrict__ w, int n, MixPdfArgs a, double *pdf, double *mom_mix, double *ratios)
+{
+    constexpr int TH = kMixBins * kMixSlices;
+    const int L = a.counts_len;
+    const int off_c = a.nq * a.nq + 2 * a.nt;
+    __shared__ double wn[1024], part[TH], mom[kNMom];
+    for (int i = threadIdx.x; i < n; i += TH) {
+        const double npts = (double)counts[(long long)i * L + off_c + 6];
+        wn[i] = npts > 0.0 ? w[i] / npts : 0.0;
+    }
+    __syncthreads();
+    if (blockIdx.x + 1 < gridDim.x) {
+        const int b = blockIdx.x * kMixBins + threadIdx.x % kMixBins, slice = threadIdx.x / kMixBins;
+        const bool in = b < mix_pdf_len(a);
+        // gradient bins follow the 8 counters; 3 longitudinal and 6
+        // transverse samples per grid point
+        const bool grad = b >= off_c;
+        double s = 0.0;
+        if (in) {
+            const unsigned long long *c = counts + (grad ? b + 8 : b);
+#pragma unroll 4
+            for (int i = slice; i < n; i += kMixSlices) s += wn[i] * (double)c[(long long)i * L];
+        }
+        part[threadIdx.x] = s;
+        __syncthreads();
+        if (slice == 0 && in) {
+            for (int k = 1; k < kMixSlices; ++k) s += part[k * kMixBins + threadIdx.x];
+            double width = b < a.nq * a.nq ? a.dq * a.dr : a.dt;
+            if (grad) width = a.dg * (b < off_c + a.ng ? 3.0 : 6.0);
+            pdf[b] = s / width;
+        }
+        return;
+    }
+    constexpr int MS = TH / kNMom;   // member slices of the moments
+    const int q = threadIdx.x % kNMom, slice = threadIdx.x / kNMom;
+    double s = 0.0;
+    if (slice < MS)
+        for (int i = slice; i < n; i += MS) s += wn[i] * moments[(long long)i * kNMom + q];
+    part[threadIdx.x] = s;
+    __syncthreads();
+    if (slice == 0) {
+        for (int k = 1; k < MS; ++k) s += part[k * kNMom + q];
+        mom[q] = s;
+        mom_mix[q] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) mix_ratios(mom, ratios);
 }
 
 // ---------------------------------------------------------------------------
@@ -393,10 +430,10 @@ void launch_mixture(const double *lam, int n, const MixWeightArgs &wa, const uns
                     const double *moments, const MixPdfArgs &pa, double *w, double *covered, double *pdf,
                     double *mom_mix, double *ratios, cudaStream_t s)
 {
-    k_mix_weights<<<1, 1024, 0, s>>>(lam, n, wa, w, covered);
+    k_mix_weights<<<1, (n + 31) / 32 * 32, 0, s>>>(lam, n, wa, w, covered);
     const int nb = mix_pdf_len(pa);
-    k_mix_pdf<<<(nb + 255) / 256, 256, 0, s>>>(counts, moments, w, n, pa, pdf, mom_mix);
-    k_mix_ratios<<<1, 32, 0, s>>>(mom_mix, ratios);
+    k_mix_pdf<<<(nb + kMixBins - 1) / kMixBins + 1, kMixBins * kMixSlices, 0, s>>>(counts, moments, w, n, pa, pdf,
+                                                                                   mom_mix, ratios);
 }
 
 }  // namespace ens

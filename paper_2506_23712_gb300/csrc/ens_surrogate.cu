@@ -450,23 +450,38 @@ __global__ void k_pack_weights(const float *p, __nv_bfloat16 *W1b, __nv_bfloat16
     }
 }
 
-// mixture of the surrogate densities over a lambda quadrature:
-// pdf(b) = sum_j w_j q(b | lambda_j) / width(b)
-__global__ void k_quad_mix(const float *q, const double *w, int nlam, int per, int nq, double dq, double dr,
-                           double dt, double *pdf)
+// mixture of the surrogate densities over a lambda quadrature: pdf(b) =
+// sum_j w_j q(b | lambda_j) / width(b); pdf[per] = *err (one copy to the host
+// brings both).  32 bins per block, the quadrature points over 8 threads per
+// bin: 110 us with a thread per bin (18 blocks), FP64 and load latency.
+__global__ void __launch_bounds__(256)
+k_quad_mix(const float *__restrict__ q, const double *__restrict__ w, int nlam, int per, int nq, double dq, double dr,
+           double dt, double *pdf, const int *err)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= per) return;
+    __shared__ double part[256];
+    const int b = blockIdx.x * 32 + (threadIdx.x & 31), slice = threadIdx.x >> 5;
     double s = 0.0;
-    for (int j = 0; j < nlam; ++j) s += w[j] * (double)q[(long long)j * per + b];
-    pdf[b] = s / (b < nq * nq ? dq * dr : dt);
+    if (b < per) {
+#pragma unroll 8
+        for (int j = slice; j < nlam; j += 8) s += w[j] * (double)q[(long long)j * per + b];
+    }
+    part[threadIdx.x] = s;
+    __syncthreads();
+    if (slice == 0 && b < per) {
+        for (int k = 1; k < 8; ++k) s += part[32 * k + threadIdx.x];
+        pdf[b] = s / (b < nq * nq ? dq * dr : dt);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) pdf[per] = (double)*err;
 }
 
 __global__ void k_quad_weights(double lo, double hi, int n, int kind, double c, double Z, double mu, double sigma,
                                double *lam, double *w)
 {
     // midpoint rule over [lo, hi]; cell masses of the lambda distribution
-    __shared__ double tot;
+    // (one block of whole warps; the masses added up by a tree: one thread
+    // adding them took 40 us for 512 points)
+    __shared__ double scratch[32];
+    double sum = 0.0;
     const double d = (hi - lo) / n;
     const double m = kind == 0 ? -4.5 * c * Z : mu;
     const double s = kind == 0 ? sqrt(9.0 * c * Z) : sigma;
@@ -476,14 +491,13 @@ __global__ void k_quad_weights(double lo, double hi, int n, int kind, double c, 
         const double za = (a - m) / s, zb = (b - m) / s;
         w[j] = za >= 0.0 ? 0.5 * (erfc(za * 0.70710678118654752440) - erfc(zb * 0.70710678118654752440))
                          : 0.5 * (erfc(-zb * 0.70710678118654752440) - erfc(-za * 0.70710678118654752440));
+        sum += w[j];
     }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = sum;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int j = 0; j < n; ++j) t += w[j];
-        tot = t;
-    }
-    __syncthreads();
+    double tot = 0.0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) tot += scratch[k];
     for (int j = threadIdx.x; j < n; j += blockDim.x) w[j] = tot > 0.0 ? w[j] / tot : 0.0;
 }
 
@@ -1125,7 +1139,7 @@ ens_status ens_surrogate_create(uint64_t seed, void *stream, ens_surrogate **out
          cudaMalloc(&S->lam5, sizeof(uint32_t) * 4096) == cudaSuccess &&
          cudaMalloc(&S->bias, sizeof(MlpBias)) == cudaSuccess &&
          cudaMalloc(&S->err, sizeof(int)) == cudaSuccess && cudaMalloc(&S->wq, sizeof(double) * 4096) == cudaSuccess &&
-         cudaMalloc(&S->pdf, sizeof(double) * 1 << 20) == cudaSuccess &&
+         cudaMalloc(&S->pdf, sizeof(double) * ((1 << 20) + 1)) == cudaSuccess &&
          cudaMalloc(&S->img, 32768 + 2 * 131072) == cudaSuccess &&
          train_prepare() == cudaSuccess;
     int dev = 0;
@@ -1302,21 +1316,20 @@ ens_status ens_surrogate_mixture(ens_surrogate *S, const ens_hist_spec *h, const
     const long long real = (long long)nquad * rs.per_member, rows = pad128(real);
     if (rs.per_member > (1 << 20)) return ENS_EINVAL;
     if (!alloc_rows(S, rs, rows, 3 * nquad)) return ENS_ENOMEM;
-    k_quad_weights<<<1, 256, 0, S->s>>>(lam_lo, lam_hi, nquad, w->kind, w->c, w->Z, w->mu, w->sigma, S->lam, S->wq);
+    k_quad_weights<<<1, 512, 0, S->s>>>(lam_lo, lam_hi, nquad, w->kind, w->c, w->Z, w->mu, w->sigma, S->lam, S->wq);
     if (!forward_fused(S, rs, real)) return ENS_ECUDA;
     k_softmax_ce<<<3 * nquad, 256, 0, S->s>>>(S->logit.as<float>(), nullptr, rs.nq, rs.nt, 1.0, S->q.as<float>(),
                                              nullptr, nullptr);
     const double dq = 2.0 * h->q_lim / h->qr_bins, dr = 2.0 * h->r_lim / h->qr_bins;
     const double dt = (h->tail_hi - h->tail_lo) / h->tail_bins;
-    k_quad_mix<<<blocks(rs.per_member, 256), 256, 0, S->s>>>(S->q.as<float>(), S->wq, nquad, rs.per_member, rs.nq, dq, dr, dt,
-                                                             S->pdf);
+    k_quad_mix<<<blocks(rs.per_member, 32), 256, 0, S->s>>>(S->q.as<float>(), S->wq, nquad, rs.per_member, rs.nq, dq,
+                                                            dr, dt, S->pdf, S->err);
     if (cudaGetLastError() != cudaSuccess) return ENS_ECUDA;
-    std::vector<double> pdf(rs.per_member);
-    if (cudaMemcpyAsync(pdf.data(), S->pdf, sizeof(double) * rs.per_member, cudaMemcpyDeviceToHost, S->s) !=
-        cudaSuccess)
+    std::vector<double> pdf(rs.per_member + 1);
+    if (cudaMemcpyAsync(pdf.data(), S->pdf, sizeof(double) * pdf.size(), cudaMemcpyDeviceToHost, S->s) != cudaSuccess ||
+        cudaStreamSynchronize(S->s) != cudaSuccess)
         return ENS_ECUDA;
-    ens_status st = check_err(S);
-    if (st != ENS_OK) return st;
+    if (pdf[rs.per_member] != 0.0) return ENS_ETIMEOUT;
     const int nq2 = rs.nq * rs.nq;
     if (out->pdf_qr) std::memcpy(out->pdf_qr, pdf.data(), sizeof(double) * nq2);
     if (out->pdf_eps) std::memcpy(out->pdf_eps, pdf.data() + nq2, sizeof(double) * rs.nt);
@@ -1379,7 +1392,7 @@ ens_status ens_surrogate_time_infer(ens_surrogate *S, const ens_hist_spec *h, in
     RowSpec rs{h->qr_bins, h->tail_bins, h->qr_bins * h->qr_bins + 2 * h->tail_bins};
     const long long real = (long long)nquad * rs.per_member, rows = pad128(real);
     if (!alloc_rows(S, rs, rows, 3 * nquad)) return ENS_ENOMEM;
-    k_quad_weights<<<1, 256, 0, S->s>>>(-5.0, 5.0, nquad, 1, 0.0, 0.0, 0.0, 1.0, S->lam, S->wq);
+    k_quad_weights<<<1, 512, 0, S->s>>>(-5.0, 5.0, nquad, 1, 0.0, 0.0, 0.0, 1.0, S->lam, S->wq);
     if (!host_bias(S)) return ENS_ECUDA;
     feature_table(S, rs, nquad);
     auto launch = [&]() { launch_infer(S, rs, real, nullptr); };

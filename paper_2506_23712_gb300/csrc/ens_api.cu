@@ -518,11 +518,12 @@ static ens_status init_context(ens_ctx *ctx, const ens_member_desc *m, int n, co
                      gr.geo.N, need, smem_optin);
             return fail(ctx, ENS_EINVAL, buf);
         }
-        ENS_CUDA(ctx, prepare_kernels(gr.geo.N, h->qr_bins, h->tail_bins, h->grad_bins));
+        ENS_CUDA(ctx, prepare_kernels(gr.geo.N, smem_optin));
         const int per_sm = znl_ctas_per_sm(gr.geo.N);
         if (per_sm <= 0 || ctx->sms <= 0) return fail(ctx, ENS_ECUDA, "occupancy query of the z pass failed");
         gr.geo.z_ctas = per_sm * ctx->sms;
         gr.geo.sms = ctx->sms;
+        gr.geo.smem_optin = smem_optin;
         launch_twiddles(const_cast<float2 *>(gr.geo.tw), gr.geo.N, st);
         ENS_CUDA(ctx, cudaMemsetAsync(gr.geo.U, 0, sizeof(float2) * 3 * gr.geo.sU * gr.geo.members, st));
         ENS_CUDA(ctx, cudaMemsetAsync(gr.geo.S, 0, sizeof(float2) * 3 * gr.geo.sU * gr.geo.members, st));
@@ -893,14 +894,13 @@ ens_status ens_gradient_stats(ens_ctx *ctx, int accumulate)
     if (!accumulate) {
         ENS_CUDA(ctx, cudaMemsetAsync(ctx->counts, 0, sizeof(unsigned long long) * n * L, st));
     }
-    ENS_CUDA(ctx, cudaMemsetAsync(ctx->mom_partial, 0, sizeof(double) * n * ctx->mom_blocks * kNMom, st));
     for (auto &gr : ctx->groups) {
         const Geo &g = gr.geo;
         launch_pass(Pass::IX, 1, g, ctx->md, nullptr, 0, 0, 0, st);
         launch_pass(Pass::IY, kIYGrad, g, ctx->md, nullptr, 0, 0, 6, st);
         launch_pass(Pass::ZSTAT, 0, g, ctx->md, &ctx->hd, 0, 0, 0, st);
+        launch_finish_stats(g, ctx->moments, accumulate, st);
     }
-    launch_finish_stats(ctx->mom_partial, ctx->mom_blocks, ctx->moments, n, accumulate, st);
     ENS_CUDA(ctx, cudaGetLastError());
     return ENS_OK;
 }

@@ -60,6 +60,7 @@ struct Geo {
                                  // 2 fused with the two halves in overlapping warp groups
     int z_mode;                  // 0: persistent TMA z pass, 1: one CTA per row group
     int z_ctas;                  // persistent CTAs of the z-direction nonlinear pass
+    int smem_optin;              // shared memory a CTA may ask for
     int sms;                     // streaming multiprocessors of the device (persistent launches)
     // failure test only (ens_test_skip_copy): the persistent z pass issues no
     // bulk copy for the first row group of this member (local index in the

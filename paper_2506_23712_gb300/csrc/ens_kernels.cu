@@ -116,14 +116,22 @@ __global__ void k_edges(float *eq, float *er, float *et, float *eg, int nq, int 
         et[b] = (float)pow(10.0, t_lo + (t_hi - t_lo) * (double)b / (double)nt);
 }
 
-__global__ void k_finish_stats(const double *mom_partial, int blocks, double *moments, int accumulate)
+// one block of kNMom x 8 threads per member: the partial moments of its blocks
+constexpr int kFinishSlices = 8;
+__global__ void __launch_bounds__(kNMom * kFinishSlices)
+k_finish_stats(const double *__restrict__ mom_partial, int stride, int blocks, double *moments, int first,
+               int accumulate)
 {
-    const int gm = blockIdx.x, t = threadIdx.x;
-    if (t >= kNMom) return;
+    const int gm = first + blockIdx.x, q = threadIdx.x % kNMom, slice = threadIdx.x / kNMom;
+    __shared__ double part[kNMom * kFinishSlices];
     double s = 0.0;
-    const double *pp = mom_partial + (long long)gm * blocks * kNMom;
-    for (int b = 0; b < blocks; ++b) s += pp[(long long)b * kNMom + t];
-    moments[gm * kNMom + t] = accumulate ? moments[gm * kNMom + t] + s : s;
+    const double *pp = mom_partial + (long long)gm * stride * kNMom;
+    for (int b = slice; b < blocks; b += kFinishSlices) s += pp[(long long)b * kNMom + q];
+    part[threadIdx.x] = s;
+    __syncthreads();
+    if (slice != 0) return;
+    for (int k = 1; k < kFinishSlices; ++k) s += part[k * kNMom + q];
+    moments[gm * kNMom + q] = accumulate ? moments[gm * kNMom + q] + s : s;
 }
 
 // ---------------------------------------------------------------------------
@@ -323,7 +331,7 @@ size_t stats_smem(int N, int nq, int nt, int ng)
 
 int stats_blocks(int N)
 {
-#define X(n) if (N == n) return stats_ctas<n>();
+#define X(n) if (N == n) return stats_ctas<n>() * kStatsMaxSub;
     ENS_SUPPORTED_N(X)
 #undef X
     return 0;
@@ -337,10 +345,10 @@ const SizedOps *sized_ops(int N)
     return nullptr;
 }
 
-cudaError_t prepare_kernels(int N, int nq, int nt, int ng)
+cudaError_t prepare_kernels(int N, int smem_optin)
 {
     const SizedOps *o = sized_ops(N);
-    return o ? o->prepare(nq, nt, ng) : cudaErrorInvalidValue;
+    return o ? o->prepare(smem_optin) : cudaErrorInvalidValue;
 }
 
 bool plan_variant_available(int N) { return has_plan_variant(N); }
@@ -420,10 +428,13 @@ void launch_bin_check(const HistDev &h, int axis, const float *x, int n, int *ou
     if (n > 0) k_bin_check<<<(n + 255) / 256, 256, 0, s>>>(h, axis, x, n, out);
 }
 
-void launch_finish_stats(const double *mom_partial, int blocks, double *moments, int nmembers, int accumulate,
-                         cudaStream_t s)
+void launch_finish_stats(const Geo &g, double *moments, int accumulate, cudaStream_t s)
 {
-    k_finish_stats<<<nmembers, 64, 0, s>>>(mom_partial, blocks, moments, accumulate);
+    const SizedOps *o = sized_ops(g.N);
+    if (!o) return;
+    k_finish_stats<<<g.members, kNMom * kFinishSlices, 0, s>>>(g.mom_partial, g.mom_blocks,
+                                                               o->stats_used(g.members, g.sms), moments, g.first,
+                                                               accumulate);
 }
 
 void launch_mixture(const double *lam, int n, const MixWeightArgs &wa, const unsigned long long *counts,

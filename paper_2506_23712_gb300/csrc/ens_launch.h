@@ -29,9 +29,9 @@ __host__ __device__ inline int mix_pdf_len(const MixPdfArgs &a) { return a.nq * 
 
 bool supported_n(int N);
 int plan_threads(int N);
-int stats_blocks(int N);
+int stats_blocks(int N);   // most partial-moment blocks per member
 size_t stats_smem(int N, int nq, int nt, int ng);   // shared memory per CTA of the statistics pass
-cudaError_t prepare_kernels(int N, int nq, int nt, int ng);
+cudaError_t prepare_kernels(int N, int smem_optin);
 int znl_ctas_per_sm(int N, int var = 0);   // resident CTAs per SM of the persistent z pass (0 on error)
 bool zplan_variant_available(int N);       // the persistent z pass has a second warp plan for this size
 bool plan_variant_available(int N);   // the x passes have a second FFT plan for this size
@@ -39,11 +39,12 @@ bool fx_ws_available(int N);          // the last pass has its warp-group varian
 
 // Pass launchers of one grid size (ens_sized.cu, one translation unit per N).
 struct SizedOps {
-    cudaError_t (*prepare)(int nq, int nt, int ng);
+    cudaError_t (*prepare)(int smem_optin);
     int (*znl_ctas_per_sm)(int var);
     void (*launch)(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, int stage, int last,
                    int arg, cudaStream_t s);
     bool (*fx_ws)();   // the warp-group variant of the last pass exists for this size
+    int (*stats_used)(int members, int sms);   // partial-moment blocks per member of a snapshot
 };
 template <int N>
 const SizedOps *sized_ops_for();
@@ -77,8 +78,8 @@ void launch_ic(const Geo &g, MemberDev *md, cudaStream_t s);
 void launch_twiddles(float2 *tw, int N, cudaStream_t s);
 void launch_edges(float *eq, float *er, float *et, float *eg, int nq, int nt, int ng, double q_lim, double r_lim,
                   double t_lo, double t_hi, double g_lim, cudaStream_t s);
-void launch_finish_stats(const double *mom_partial, int blocks, double *moments, int nmembers, int accumulate,
-                         cudaStream_t s);
+// moment sums of a group's members from their partial-moment blocks
+void launch_finish_stats(const Geo &g, double *moments, int accumulate, cudaStream_t s);
 void launch_bin_check(const HistDev &h, int axis, const float *x, int n, int *out, cudaStream_t s);
 void launch_mixture(const double *lam, int n, const MixWeightArgs &wa, const unsigned long long *counts,
                     const double *moments, const MixPdfArgs &pa, double *w, double *covered, double *pdf,

@@ -48,7 +48,7 @@ cudaError_t prepare_variants()
     return e;
 }
 
-cudaError_t prepare(int nq, int nt, int ng)
+cudaError_t prepare(int smem_optin)
 {
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
@@ -72,7 +72,7 @@ cudaError_t prepare(int nq, int nt, int ng)
     chk(allow_smem(k_z<N, 1>, smem_rows<N>()));
     chk(allow_smem(k_z<N, 3>, smem_rows<N>()));
     chk(allow_smem(k_z<N, 4>, smem_rows<N>()));
-    chk(allow_smem(k_z_stats<N>, smem_stats<N>(nq, nt, ng)));
+    chk(cudaFuncSetAttribute(k_z_stats<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin));
     chk(allow_smem(k_znl<N>, ZCfg<N>::smem_bytes()));
     return e;
 }
@@ -224,8 +224,12 @@ void launch(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, 
         }
         break;
     case Pass::ZSTAT: {
-        const dim3 grid((unsigned)stats_ctas<N>(), g.members);
-        k_z_stats<N><<<grid, 32 * SCfg<N>::WPB, smem_stats<N>(h->nq, h->nt, h->ng), s>>>(g, *h, md);
+        const int sub = stats_sub<N>(g.members, g.sms), warps = stats_warps<N>(sub);
+        const size_t base = smem_stats<N>(h->nq, h->nt, h->ng, warps);
+        const int copies =
+            stats_split<N>() ? grad_copies(h->ng, (size_t)g.smem_optin > base ? g.smem_optin - base : 0) : 1;
+        const size_t smem = base + (copies > 1 ? sizeof(unsigned) * (size_t)(copies * grad_pitch(h->ng)) : 0);
+        k_z_stats<N><<<dim3(stats_ctas<N>() * sub, g.members), 32 * warps, smem, s>>>(g, *h, md, sub, copies);
         break;
     }
     }
@@ -233,7 +237,9 @@ void launch(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, 
 
 bool fx_ws() { return has_fx_ws<N>(); }
 
-const SizedOps kOps = {prepare, znl_per_sm, launch, fx_ws};
+int stats_used(int members, int sms) { return stats_ctas<N>() * stats_sub<N>(members, sms); }
+
+const SizedOps kOps = {prepare, znl_per_sm, launch, fx_ws, stats_used};
 
 }  // namespace
 

@@ -12,16 +12,22 @@
 // bin b iff edge[b] <= x < edge[b+1] on FP32 edges (the floor of the affine
 // or log map's estimate, corrected once against the edge table, so the
 // decision is exactly the edge comparison).  Counts go to per-CTA shared-memory
-// histograms (plain shared atomics for the Q-R and tail histograms,
-// warp-aggregated increments for the gradient components), flushed to the
-// member's uint64 counts once per CTA.  Moments: FP32 sums per thread
+// histograms (plain shared atomics; the gradient components, nine increments
+// per point into a few crowded bins, into several copies of their histograms
+// picked by lane where they fit), flushed to the member's uint64 counts once
+// per CTA.  Moments: FP32 sums per thread
 // (packed FP32x2 for the component pairs) over up to kStatsFlush rows, warp
 // shuffle reduction into FP64 per warp, FP64 fixed-order reduction across
 // warps and CTAs.
 //
-// Layout of the work: grid (stats_ctas<N>(), members); CTA c of member m
-// takes a contiguous block of rows, its warps stream over the row groups of
-// the block (32/P rows per group).  A warp stages the eight half-spectrum
+// Layout of the work: a member's rows are cut into stats_ctas<N>() contiguous
+// blocks, the row groups of a block (32/P rows each) dealt out to WPB streams
+// (group g to stream g mod WPB), and a stream's groups into units of
+// kStatsFlush, the length of an FP32 moment sum.  A unit is always summed by
+// one warp in the same order, whichever CTA runs it, so the split may follow
+// the number of members: one CTA of WPB warps per block where the blocks fill
+// the chip, else `sub` CTAs per block with a share of its units each
+// (stats_sub: 16 x 64^3 members have 32 blocks for 152 SMs).  A warp stages the eight half-spectrum
 // rows of a group in shared memory (cp.async.bulk, TMA; zero past the kept
 // modes), reads them into registers, and refills the same buffer with the
 // next group while it transforms and bins the current one (the work per
@@ -68,12 +74,6 @@ __device__ __forceinline__ int bin_log(float x, BinMap m, const float *e, int n)
     return bin_tab(x, fmaf(__log2f(x), m.a, m.c), e, n);
 }
 
-// increment of hist[key] without aggregation (key < 0: none)
-__device__ __forceinline__ void lane_count(unsigned *hist, int key)
-{
-    if (key >= 0) atomicAdd(&hist[key], 1u);
-}
-
 // warp-aggregated increment of hist[key] (key < 0: no increment)
 __device__ __forceinline__ void warp_count(unsigned *hist, int key)
 {
@@ -82,12 +82,21 @@ __device__ __forceinline__ void warp_count(unsigned *hist, int key)
     if (key >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[key], (unsigned)__popc(peers));
 }
 
+// increment of hist[key] without aggregation (key < 0: none)
+__device__ __forceinline__ void lane_count(unsigned *hist, int key)
+{
+    if (key >= 0) atomicAdd(&hist[key], 1u);
+}
+
 __device__ __forceinline__ float warp_sum(float v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+
+// moment partials are flushed from FP32 registers to FP64 every kStatsFlush row groups
+constexpr int kStatsFlush = 32;
 
 // Shape of the statistics pass: warps per CTA, staged row pitch, CTAs per member.
 template <int N>
@@ -110,22 +119,67 @@ struct SCfg {
     // CTAs per member: a power of two up to 32, at least 32 row groups per warp
     static constexpr int pow2_floor(int x) { return x >= 32 ? 32 : x >= 16 ? 16 : x >= 8 ? 8 : x >= 4 ? 4 : x >= 2 ? 2 : 1; }
     static constexpr int CTAS = pow2_floor(GROUPS / (WPB * 32));
-    static_assert(GROUPS % CTAS == 0, "row groups split evenly over the CTAs of a member");
+    static_assert(GROUPS % CTAS == 0, "row groups split evenly over the blocks of a member");
+    static constexpr int GPB = GROUPS / CTAS;                                // row groups of a block
+    static constexpr int SEG = ((GPB + WPB - 1) / WPB + kStatsFlush - 1) / kStatsFlush;   // units per stream
+    static constexpr int UNITS = WPB * SEG;                                  // units of a block
 };
 
-// moment partials are flushed from FP32 registers to FP64 every kStatsFlush row groups
-constexpr int kStatsFlush = 32;
+// 256^3 keeps one CTA per block of rows, warp w running stream w, and one
+// histogram copy: the compiler decides by the code around them which products
+// of Tr A^2 and Tr S^2 it contracts, and with 16 warps on 128 registers every
+// change of the loop moved some of those roundings, hence a few counts at bin
+// edges (4 in 3.4e8 points).  The other sizes kept all of them.
+template <int N>
+__host__ __device__ constexpr bool stats_split() { return N != 256; }
+
+// CTAs per block of rows: enough for four rounds over the SMs, at most
+// kStatsMaxSub (and one unit each).  More CTAs than that cost more in clearing
+// and flushing their histograms than the better balance gives.
+constexpr int kStatsMaxSub = 12;
+template <int N>
+int stats_sub(int members, int sms)
+{
+    if (!stats_split<N>()) return 1;
+    const long long blocks = (long long)SCfg<N>::CTAS * members;
+    int sub = (int)((4LL * sms + blocks - 1) / blocks);
+    sub = sub < 1 ? 1 : sub > kStatsMaxSub ? kStatsMaxSub : sub;
+    return sub > SCfg<N>::UNITS ? SCfg<N>::UNITS : sub;
+}
+// warps of such a CTA
+template <int N>
+int stats_warps(int sub)
+{
+    const int units = (SCfg<N>::UNITS + sub - 1) / sub;
+    return units < SCfg<N>::WPB ? units : SCfg<N>::WPB;
+}
 
 template <int N>
 constexpr int stats_ctas() { return SCfg<N>::CTAS; }
 
 template <int N>
-constexpr size_t smem_stats(int nq, int nt, int ng)
+constexpr size_t smem_stats(int nq, int nt, int ng, int warps = SCfg<N>::WPB)
 {
     using C = SCfg<N>;
-    return sizeof(float2) * (size_t)(N + C::LT) + sizeof(uint64_t) * 2 * C::WPB + sizeof(float2) * (size_t)C::WPB * C::STAGE +
-           sizeof(float2) * (size_t)C::WPB * C::LPW * C::SROW + sizeof(double) * C::WPB * kNMom +
+    return sizeof(float2) * (size_t)(N + C::LT) + sizeof(uint64_t) * 2 * warps + sizeof(float2) * (size_t)warps * C::STAGE +
+           sizeof(float2) * (size_t)warps * C::LPW * C::SROW + sizeof(double) * warps * kNMom +
            sizeof(unsigned) * (size_t)counts_len_of(nq, nt, ng) + sizeof(float) * (2 * (nq + 1) + nt + 1 + ng + 1) + 16;
+}
+
+// Copies of the gradient-component histograms (2 ng bins and 4 counters, an
+// odd pitch): the nine components of a point fall into a handful of bins, so
+// 32 lanes on one copy wait on each other; lane l counts in copy l mod copies.
+// At most 8, and no more than the shared memory left beside the rest holds
+// (`room` bytes), down to one, which is the member's histogram layout itself.
+// 16 x 64^3 with 128 bins, whole snapshot: 1006 us with one copy, increments
+// aggregated by warp, and 32 CTAs; 431 us with 8 copies and 384 CTAs.
+__host__ __device__ inline int grad_pitch(int ng) { return 2 * ng + 5; }
+inline int grad_copies(int ng, size_t room)
+{
+    if (ng <= 0) return 1;
+    int c = 8;
+    while (c > 1 && sizeof(unsigned) * (size_t)(c * grad_pitch(ng)) > room) c >>= 1;
+    return c;
 }
 
 // packed FP32x2 helpers for the moment sums
@@ -144,11 +198,13 @@ __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c)
 
 template <int N>
 __global__ void __launch_bounds__(32 * SCfg<N>::WPB, 1)
-k_z_stats(Geo g, HistDev h, const MemberDev *md)
+k_z_stats(Geo g, HistDev h, const MemberDev *md, int sub, int copies)
 {
     using C = SCfg<N>;
     using PI = WPlanInfo<N>;
-    constexpr int P = C::P, V = C::V, LPW = C::LPW, NZ2 = C::NZ2, WPB = C::WPB;
+    constexpr bool SPLIT = stats_split<N>();
+    constexpr int P = C::P, V = C::V, LPW = C::LPW, NZ2 = C::NZ2;
+    const int WPB = SPLIT ? blockDim.x >> 5 : C::WPB;   // warps of this CTA
     extern __shared__ __align__(16) unsigned char smraw[];
     float2 *tw = reinterpret_cast<float2 *>(smraw);
     float2 *ltw = tw + N;   // lane-major inter-pass twiddles (padded plans)
@@ -162,12 +218,15 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
     float *er = eq + (h.nq + 1);
     float *et = er + (h.nq + 1);
     float *eg = et + (h.nt + 1);
+    unsigned *gh = reinterpret_cast<unsigned *>(eg + (h.ng + 1));   // [copies][grad_pitch] (copies > 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int line = lane / P, p = lane % P;
     uint64_t *bar = bars + 2 * warp;
     float2 *st = stage + warp * C::STAGE;
     float2 *rowbuf = rows + warp * LPW * C::SROW;
     for (int i = threadIdx.x; i < L; i += blockDim.x) hist[i] = 0u;
+    if (SPLIT && copies > 1)
+        for (int i = threadIdx.x; i < copies * grad_pitch(h.ng); i += blockDim.x) gh[i] = 0u;
     for (int i = threadIdx.x; i <= h.nq; i += blockDim.x) {
         eq[i] = h.edges_q[i];
         er[i] = h.edges_r[i];
@@ -189,8 +248,26 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
 
     const int m = blockIdx.y;
     const float nu = (float)md[g.first + m].nu;
-    constexpr int GPC = C::GROUPS / C::CTAS;   // row groups of this CTA
-    const long long g0 = (long long)blockIdx.x * GPC;
+    constexpr int GPB = C::GPB;
+    const int blk = SPLIT ? blockIdx.x / sub : blockIdx.x, part = SPLIT ? blockIdx.x % sub : 0;
+    const long long g0 = (long long)blk * GPB;
+    // SPLIT: this warp's units [u, u1), a contiguous share of the CTA's share of
+    // the block; k: its current row group, left: groups of the unit from k on
+    int u = 0, u1 = 0, left = 0, k = warp;
+    auto begin = [&]() {   // first group of the next unit that has any
+        for (; u < u1; ++u) {
+            k = u / C::SEG + (u % C::SEG) * kStatsFlush * C::WPB;
+            left = min(kStatsFlush, (GPB - k + C::WPB - 1) / C::WPB);
+            if (k < GPB) return;
+        }
+    };
+    if constexpr (SPLIT) {
+        const int ua = part * C::UNITS / sub, ub = (part + 1) * C::UNITS / sub;
+        u = ua + warp * (ub - ua) / WPB;
+        u1 = ua + (warp + 1) * (ub - ua) / WPB;
+        begin();
+    }
+    auto more = [&]() { return SPLIT ? u < u1 : k < GPB; };
     const uint32_t bytes = (uint32_t)(LPW * 8 * NZ2 * sizeof(float2));
     const float2 *Bm = g.B + (long long)m * kFields * Dims<N>::SB;
     auto issue = [&](int k) {   // lane 0: row group g0 + k
@@ -204,14 +281,15 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
                 bulk_g2s(dst + (l * 8 + f) * C::PITCH, src + f * Dims<N>::SB + l * Dims<N>::NZP,
                          NZ2 * (uint32_t)sizeof(float2), &bar[0]);
     };
-    int k = warp;
-    if (lane == 0 && k < GPC) issue(k);
+    if (lane == 0 && more()) issue(k);
 
     auto at = [&](int pos) { return row_slot<N>(rowbuf, line, pos); };
     float2 *myrow = rowbuf + line * C::SROW;
     const int off_e = h.nq * h.nq, off_w = off_e + h.nt, off_c = off_w + h.nt;
     const BinMap mq = lin_map(h.q_lo, h.q_inv_w), mr = lin_map(h.r_lo, h.r_inv_w);
     const BinMap mt = log_map(h.t_lo, h.t_inv_w), mg = lin_map(h.g_lo, h.g_inv_w);
+    // gradient components: keys 0 .. 2 ng + 3 (longitudinal, transverse, counters) of this lane's copy
+    unsigned *const mygh = copies > 1 ? gh + (lane & (copies - 1)) * grad_pitch(h.ng) : hist + off_c + 8;
     const int off_gl = off_c + 8, off_gt = off_gl + h.ng, off_gc = off_gt + h.ng;
 
     // FP32 moment partials: component pairs (2q, 2q + 1) packed, A_33 alone,
@@ -247,7 +325,7 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
 
     bool timed_out = false;
     int it = 0;
-    for (; k < GPC; ++it, k += WPB) {
+    for (; more(); ++it) {
         if (!mbar_wait_warp(&bar[0], (uint32_t)(it & 1))) {
             timed_out = true;
             break;
@@ -258,9 +336,18 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
 #pragma unroll
         for (int q = 0; q < 4; ++q) PairSlots<N, 0, 0>::load(v[q], X + 2 * q * R, X + (2 * q + 1) * R, p);
         __syncwarp();   // staged rows read: the buffer takes the next group
-        if (lane == 0 && k + WPB < GPC) {
+        k += C::WPB;
+        bool unit_end = false;
+        if constexpr (SPLIT) {
+            unit_end = --left == 0;
+            if (unit_end) {
+                ++u;
+                begin();
+            }
+        }
+        if (lane == 0 && more()) {
             fence_proxy_async_smem();   // the reads above precede the refill
-            issue(k + WPB);
+            issue(k);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -310,13 +397,23 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
 #pragma unroll
                 for (int c = 0; c < 9; ++c) {
                     int kg = -1;
-                    if (finite) {
-                        const int bg = bin_lin(A[c] * h.g_scale, mg, eg, h.ng);
-                        const bool lon = c % 4 == 0;
-                        kg = bg < 0 ? off_gc + (lon ? 0 : 2)
-                                    : (bg >= h.ng ? off_gc + (lon ? 1 : 3) : (lon ? off_gl : off_gt) + bg);
+                    if constexpr (SPLIT) {
+                        if (finite) {
+                            const int bg = bin_lin(A[c] * h.g_scale, mg, eg, h.ng);
+                            const bool lon = c % 4 == 0;
+                            kg = bg < 0 ? 2 * h.ng + (lon ? 0 : 2)
+                                        : (bg >= h.ng ? 2 * h.ng + (lon ? 1 : 3) : (lon ? 0 : h.ng) + bg);
+                        }
+                        lane_count(mygh, kg);
+                    } else {
+                        if (finite) {
+                            const int bg = bin_lin(A[c] * h.g_scale, mg, eg, h.ng);
+                            const bool lon = c % 4 == 0;
+                            kg = bg < 0 ? off_gc + (lon ? 0 : 2)
+                                        : (bg >= h.ng ? off_gc + (lon ? 1 : 3) : (lon ? off_gl : off_gt) + bg);
+                        }
+                        warp_count(hist, kg);
                     }
-                    warp_count(hist, kg);
                 }
             }
             // moments of the components: sums of A_c^p, p = 2, 3, 4, 6
@@ -336,22 +433,30 @@ k_z_stats(Geo g, HistDev h, const MemberDev *md)
             T4 = fmaf(b2, b2, T4);
             T6 = fmaf(b2 * b2, b2, T6);
         }
-        if ((it + 1) % kStatsFlush == 0) flush();
+        if constexpr (SPLIT) {
+            if (unit_end) flush();
+        } else {
+            if ((it + 1) % kStatsFlush == 0) flush();
+        }
     }
-    flush();
+    if constexpr (!SPLIT) flush();
     if (timed_out) {
         if (lane == 0) atomicOr(const_cast<int *>(&md[g.first + m].flags), kFlagTimeout);
         mbar_wait_warp(&bar[0], (uint32_t)(it & 1));   // the copy in flight, once more (bounded)
     }
     __syncthreads();
     unsigned long long *cnt = g.counts + (long long)(g.first + m) * L;
-    for (int i = threadIdx.x; i < L; i += blockDim.x)
-        if (hist[i]) atomicAdd(&cnt[i], (unsigned long long)hist[i]);
-    if (threadIdx.x == 0) atomicAdd(&cnt[off_c + 6], (unsigned long long)GPC * LPW * N);
-    if (threadIdx.x < kNMom) {
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+        unsigned c = hist[i];
+        if (SPLIT && copies > 1 && i >= off_c + 8)
+            for (int q = 0; q < copies; ++q) c += gh[q * grad_pitch(h.ng) + i - (off_c + 8)];
+        if (c) atomicAdd(&cnt[i], (unsigned long long)c);
+    }
+    if (threadIdx.x == 0 && part == 0) atomicAdd(&cnt[off_c + 6], (unsigned long long)GPB * LPW * N);
+    for (int q = threadIdx.x; q < kNMom; q += blockDim.x) {
         double s = 0.0;
-        for (int w = 0; w < WPB; ++w) s += wmom[w * kNMom + threadIdx.x];
-        g.mom_partial[((long long)(g.first + m) * g.mom_blocks + blockIdx.x) * kNMom + threadIdx.x] = s;
+        for (int w = 0; w < WPB; ++w) s += wmom[w * kNMom + q];
+        g.mom_partial[((long long)(g.first + m) * g.mom_blocks + blockIdx.x) * kNMom + q] = s;
     }
 }
 

@@ -264,8 +264,9 @@ typedef struct {
     double ms_per_step;  /* ens_autotune: mean step time of the winner, else 0 */
     int trials;          /* ens_autotune: configurations timed */
 } ens_tuning;
-/* Current tuning (defaults at creation: tiles 16, persistent z pass at its
- * occupancy limit, parallel groups). */
+/* Current tuning.  At creation: tiles 16 (tile_x 8 for N >= 384), persistent z
+ * pass at its occupancy limit (z_variant 2 where it exists, else 0), fx_split 1
+ * for N >= 256, parallel groups unless one of them has N >= 256. */
 ens_status ens_get_tuning(const ens_ctx *ctx, ens_tuning *out);
 /* Install a tuning (for instance one cached from an earlier ens_autotune on
  * the same device and member set).  ENS_EINVAL (not sticky, previous tuning

@@ -168,6 +168,44 @@ ens_status validate(const ens_member_desc *m, int n, const ens_hist_spec *h, std
     return validate_hist(h, why);
 }
 
+// Pass variants of a new context (ens_autotune looks for better ones).
+//   last pass      split from 256^3 on: its transform and its update each run at
+//                  the copy rate, the fused pass waits on its state reads (1054
+//                  against 1282 us per stage at 16 x 256^3, 235 / 304 at 384^3,
+//                  544 / 750 at 512^3); below that the transformed modes are a
+//                  larger part of the traffic than the waits (128^3: 242 / 212 us
+//                  at 24 members)
+//   z pass         the two-pass warp plan where there is one (256^3: 1418
+//                  against 1600 us per stage at 16 members, 96 / 109 at one)
+//   inverse x      8 columns at 384^3 and 512^3, where a 16-column tile leaves
+//                  one CTA per SM (177 / 199 us, 403 / 449 us)
+void default_variants(Geo &g)
+{
+    g.tile_x = g.N >= 384 ? 8 : kTile;
+    g.tile_y = kTile;
+    g.plan_x = 0;
+    g.fx_split = g.N >= 256 ? 1 : 0;
+    g.z_mode = zplan_variant_available(g.N) ? 2 : 0;
+}
+// Grid sizes one after another as soon as one of them fills the GPU by itself
+// (a quarter of the uneven batch: 7.73 ms per step against 8.35 in parallel
+// branches; 16 x 64^3 + 2 x 256^3: 2.32 / 2.46), in parallel branches where all are
+// small (4 x 32^3 + 2 x 64^3: 0.150 / 0.110).
+bool default_parallel(const std::vector<Group> &groups)
+{
+    for (auto &gr : groups)
+        if (gr.geo.N >= 256) return false;
+    return true;
+}
+
+// CTAs of a group's update pass that write partial sums
+int update_partials(const Geo &g, bool persistent)
+{
+    // the persistent stage kernel runs the fused update pass on 16-column tiles
+    if (persistent || g.fx_split == 2) return g.NK * g.NZp / 16;
+    return g.fx_split ? (int)((g.sU + kUpdChunk - 1) / kUpdChunk) : g.NK * g.NZp / g.tile_x;
+}
+
 // Group members by N (ascending), carve the workspace (base == nullptr: size only).
 size_t carve(const ens_member_desc *m, int n, const ens_hist_spec *h, char *base, ens_ctx *ctx)
 {
@@ -190,10 +228,7 @@ size_t carve(const ens_member_desc *m, int n, const ens_hist_spec *h, char *base
         g.NK = 2 * g.kc + 1;
         g.NZ = g.kc + 1;
         g.NZp = (g.NZ + kTile - 1) / kTile * kTile;
-        g.tile_x = g.tile_y = kTile;
-        g.plan_x = 0;
-        g.fx_split = 0;
-        g.z_mode = 0;
+        default_variants(g);
         g.z_skip_member = -1;
         g.z_skip_wait = 0;
         g.members = (int)gr.members.size();
@@ -268,6 +303,7 @@ size_t carve(const ens_member_desc *m, int n, const ens_hist_spec *h, char *base
             }
         }
         ctx->groups = groups;
+        ctx->parallel_groups = default_parallel(groups);
     }
     return ar.off + kAlign;
 }
@@ -459,7 +495,7 @@ static ens_status init_context(ens_ctx *ctx, const ens_member_desc *m, int n, co
         x.seed = d.seed;
         x.init_energy = d.init_energy;
         const Geo &g = ctx->groups[x.group].geo;
-        x.nblk = g.NK * g.NZp / g.tile_x;   // update-pass CTAs (>= sums-kernel CTAs)
+        x.nblk = update_partials(g, false);   // update-pass CTAs (>= sums-kernel CTAs)
         x.dt = x.dt_fixed;
     }
     cudaStream_t st = ctx->stream;
@@ -519,7 +555,7 @@ static ens_status init_context(ens_ctx *ctx, const ens_member_desc *m, int n, co
             return fail(ctx, ENS_EINVAL, buf);
         }
         ENS_CUDA(ctx, prepare_kernels(gr.geo.N, smem_optin));
-        const int per_sm = znl_ctas_per_sm(gr.geo.N);
+        const int per_sm = znl_ctas_per_sm(gr.geo.N, gr.geo.z_mode == 2 ? 1 : 0);
         if (per_sm <= 0 || ctx->sms <= 0) return fail(ctx, ENS_ECUDA, "occupancy query of the z pass failed");
         gr.geo.z_ctas = per_sm * ctx->sms;
         gr.geo.sms = ctx->sms;
@@ -1342,10 +1378,7 @@ ens_status sync_nblk(ens_ctx *ctx)
 {
     for (auto &gr : ctx->groups) {
         const Geo &g = gr.geo;
-        // the persistent stage kernel runs the fused update pass on 16-column tiles
-        const int nblk = ctx->persistent || g.fx_split == 2 ? g.NK * g.NZp / 16
-                         : g.fx_split                     ? (int)((g.sU + kUpdChunk - 1) / kUpdChunk)
-                                                          : g.NK * g.NZp / g.tile_x;
+        const int nblk = update_partials(g, ctx->persistent);
         std::vector<int> v(g.members, nblk);
         ENS_CUDA(ctx, cudaMemcpy2DAsync(&ctx->md[g.first].nblk, sizeof(MemberDev), v.data(), sizeof(int),
                                         sizeof(int), g.members, cudaMemcpyHostToDevice, ctx->stream));

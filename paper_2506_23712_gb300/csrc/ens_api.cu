@@ -174,7 +174,9 @@ ens_status validate(const ens_member_desc *m, int n, const ens_hist_spec *h, std
 //                  against 1282 us per stage at 16 x 256^3, 235 / 304 at 384^3,
 //                  544 / 750 at 512^3); below that the transformed modes are a
 //                  larger part of the traffic than the waits (128^3: 242 / 212 us
-//                  at 24 members)
+//                  at 24 members), but for 64^3 from 8 members on, where the fused
+//                  pass's small CTAs wait longest (step of 16 members 269 / 290
+//                  us, of 4 members 107 / 103)
 //   z pass         the two-pass warp plan where there is one (256^3: 1418
 //                  against 1600 us per stage at 16 members, 96 / 109 at one)
 //   inverse x      8 columns at 384^3 and 512^3, where a 16-column tile leaves
@@ -184,7 +186,7 @@ void default_variants(Geo &g)
     g.tile_x = g.N >= 384 ? 8 : kTile;
     g.tile_y = kTile;
     g.plan_x = 0;
-    g.fx_split = g.N >= 256 ? 1 : 0;
+    g.fx_split = g.N >= 256 || (g.N == 64 && g.members >= 8) ? 1 : 0;
     g.z_mode = zplan_variant_available(g.N) ? 2 : 0;
 }
 // Grid sizes one after another as soon as one of them fills the GPU by itself
@@ -228,10 +230,10 @@ size_t carve(const ens_member_desc *m, int n, const ens_hist_spec *h, char *base
         g.NK = 2 * g.kc + 1;
         g.NZ = g.kc + 1;
         g.NZp = (g.NZ + kTile - 1) / kTile * kTile;
-        default_variants(g);
         g.z_skip_member = -1;
         g.z_skip_wait = 0;
         g.members = (int)gr.members.size();
+        default_variants(g);
         g.first = first;
         first += g.members;
         g.sU = (long long)g.NK * g.NK * g.NZp;
@@ -343,9 +345,13 @@ Geo single(const ens_ctx *ctx, int i)
 void record_group_stage(ens_ctx *ctx, const Geo &g, int st, int last, cudaStream_t s)
 {
     launch_pass(Pass::IX, 0, g, ctx->md, nullptr, st, last, st > 0 ? 1 : 0, s);
-    launch_pass(Pass::IY, 0, g, ctx->md, nullptr, st, last, 6, s);
-    launch_pass(Pass::Z, 0, g, ctx->md, nullptr, st, last, 0, s);
-    launch_pass(Pass::FY, 0, g, ctx->md, nullptr, st, last, 0, s);
+    if (plane_fused(g)) {
+        launch_pass(Pass::PLANE, 0, g, ctx->md, nullptr, st, last, 0, s);
+    } else {
+        launch_pass(Pass::IY, 0, g, ctx->md, nullptr, st, last, 6, s);
+        launch_pass(Pass::Z, 0, g, ctx->md, nullptr, st, last, 0, s);
+        launch_pass(Pass::FY, 0, g, ctx->md, nullptr, st, last, 0, s);
+    }
     launch_pass(Pass::FX, 0, g, ctx->md, nullptr, st, last, 0, s);
 }
 
@@ -702,7 +708,7 @@ int ens_kernels_per_step(const ens_ctx *ctx)
     if (!ctx) return 0;
     if (ctx->persistent) return ctx->rk;   // one persistent launch per stage
     int per_stage = 1;   // the per-member stage reduction
-    for (auto &gr : ctx->groups) per_stage += 5 + (gr.geo.fx_split == 1 ? 1 : 0);
+    for (auto &gr : ctx->groups) per_stage += (plane_fused(gr.geo) ? 3 : 5) + (gr.geo.fx_split == 1 ? 1 : 0);
     return ctx->rk * per_stage;
 }
 

@@ -2,6 +2,7 @@
 // and the table of per-N pass launchers (each grid size compiles in its own
 // translation unit, ens_sized.cu).
 #include "ens_launch.h"
+#include "ens_plane.cuh"
 #include "ens_stats.cuh"
 #include "ens_znl.cuh"
 
@@ -311,6 +312,13 @@ bool supported_n(int N)
     ENS_SUPPORTED_N(X)
 #undef X
     return false;
+}
+
+// The stage's middle in one launch where a plane fits (N <= 64) and the tuning
+// asks for the plain variants; the failure test needs the z pass's bulk copies.
+bool plane_fused(const Geo &g)
+{
+    return has_plane(g.N) && g.z_mode == 0 && g.tile_y == kTile && g.z_skip_member < 0;
 }
 
 int plan_threads(int N)

@@ -4,6 +4,7 @@
 #include "ens_fxsplit.cuh"
 #include "ens_fxws.cuh"
 #include "ens_launch.h"
+#include "ens_plane.cuh"
 #include "ens_stats.cuh"
 #include "ens_znl.cuh"
 
@@ -48,6 +49,13 @@ cudaError_t prepare_variants()
     return e;
 }
 
+template <int M>
+cudaError_t prepare_plane()
+{
+    if constexpr (has_plane(M)) return allow_smem(k_plane<M>, PlaneCfg<M>::smem());
+    return cudaSuccess;
+}
+
 cudaError_t prepare(int smem_optin)
 {
     cudaError_t e = cudaSuccess;
@@ -55,6 +63,7 @@ cudaError_t prepare(int smem_optin)
     chk(allow_smem(k_inv_x<N, 0, 16>, smem_x<N, 16>()));
     chk(allow_smem(k_inv_x<N, 0, 8>, smem_x<N, 8>()));
     chk(prepare_variants<N>());
+    chk(prepare_plane<N>());
     chk(allow_smem(k_fwd_x_fft<N, 16>, smem_cols<N, 16>()));
     chk(allow_smem(k_inv_x<N, 1, 16>, smem_x<N, 16>()));
     chk(allow_smem(k_inv_y<N, 16>, smem_cols<N, 16>()));
@@ -75,6 +84,12 @@ cudaError_t prepare(int smem_optin)
     chk(cudaFuncSetAttribute(k_z_stats<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin));
     chk(allow_smem(k_znl<N>, ZCfg<N>::smem_bytes()));
     return e;
+}
+
+template <int M>
+void launch_plane(const Geo &g, MemberDev *md, int stage, cudaStream_t s)
+{
+    if constexpr (has_plane(M)) k_plane<M><<<dim3(M, g.members), 32 * PlaneCfg<M>::WPB, PlaneCfg<M>::smem(), s>>>(g, md, stage);
 }
 
 template <int M>
@@ -205,6 +220,7 @@ void launch(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, 
         }
         break;
     }
+    case Pass::PLANE: launch_plane<N>(g, md, stage, s); break;
     case Pass::FX:
         switch (mode) {
         case 0:

@@ -653,28 +653,11 @@ __device__ __forceinline__ double member_dt(const MemberDev &d, int N)
     return dt;
 }
 
-// End of an RK stage for member gm (one warp, lane = 0..31): the FP64
-// partial sums of the update pass -> E, dissipation, band energy, the forcing
-// amplitude alpha = eps_inj / (2 E_B) of the next stage, the CFL step after the
-// first stage, time and step count after the last.
-__device__ __forceinline__ void finish_body(MemberDev *md, const double *partial, int partial_blocks, int stage,
-                                            int last_stage, int mode, int gm, int lane)
+// Run state of a member from the sums e, s, b (energy, dissipation, band
+// energy) of the field just written: one thread.
+__device__ __forceinline__ void finish_member(MemberDev &d, double e, double s, double b, int stage, int last_stage,
+                                              int mode)
 {
-    MemberDev &d = md[gm];
-    double e = 0.0, s = 0.0, b = 0.0;
-    const double *pp = partial + (long long)gm * partial_blocks * 4;
-    for (int k = lane; k < d.nblk; k += 32) {
-        e += pp[k * 4 + 0];
-        s += pp[k * 4 + 1];
-        b += pp[k * 4 + 2];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        e += __shfl_xor_sync(0xffffffffu, e, o);
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    if (lane != 0) return;
     if (mode == 0 && stage == 0) d.dt = member_dt(d, d.N);
     // injected power of the stage just taken: alpha(u^s) * 2 E_B(u^s)
     if (mode == 0) d.P = d.alpha * 2.0 * d.EB;
@@ -696,6 +679,30 @@ __device__ __forceinline__ void finish_body(MemberDev *md, const double *partial
         d.umax = (double)__uint_as_float(d.umax_bits[0]);
         for (int q = 0; q < 4; ++q) d.umax_bits[q] = 0u;
     }
+}
+
+// End of an RK stage for member gm (one warp, lane = 0..31): the FP64
+// partial sums of the update pass -> E, dissipation, band energy, the forcing
+// amplitude alpha = eps_inj / (2 E_B) of the next stage, the CFL step after the
+// first stage, time and step count after the last.
+__device__ __forceinline__ void finish_body(MemberDev *md, const double *partial, int partial_blocks, int stage,
+                                            int last_stage, int mode, int gm, int lane)
+{
+    MemberDev &d = md[gm];
+    double e = 0.0, s = 0.0, b = 0.0;
+    const double *pp = partial + (long long)gm * partial_blocks * 4;
+    for (int k = lane; k < d.nblk; k += 32) {
+        e += pp[k * 4 + 0];
+        s += pp[k * 4 + 1];
+        b += pp[k * 4 + 2];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) finish_member(d, e, s, b, stage, last_stage, mode);
 }
 
 template <int NW>

@@ -425,7 +425,7 @@ ens_status resum(ens_ctx *ctx)
     // partial slots the sums kernel does not write must read as zero
     ENS_CUDA(ctx, cudaMemsetAsync(ctx->partial, 0, sizeof(double) * ctx->desc.size() * ctx->partial_blocks * 4,
                                   ctx->stream));
-    for (auto &gr : ctx->groups) launch_state_sums(gr.geo, ctx->md, ctx->stream);
+    for (auto &gr : ctx->groups) launch_state_sums(gr.geo, ctx->md, update_partials(gr.geo, ctx->persistent), ctx->stream);
     launch_finish(ctx->md, (int)ctx->desc.size(), ctx->partial, ctx->partial_blocks, 0, 0, 1, ctx->stream);
     ENS_CUDA(ctx, cudaGetLastError());
     return ENS_OK;
@@ -851,7 +851,7 @@ ens_status ens_step_host(ens_ctx *ctx, const void *host_in, void *host_out, size
             ENS_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_in[ci], 0));
             // energy sums of the uploaded state, as after ens_set_state
             ENS_CUDA(ctx, cudaMemsetAsync(part, 0, sizeof(double) * cnt * PB * 4, ctx->stream));
-            launch_state_sums(g, ctx->md, ctx->stream);
+            launch_state_sums(g, ctx->md, update_partials(g, ctx->persistent), ctx->stream);
             launch_finish(md, cnt, part, PB, 0, 0, 1, ctx->stream);
             for (int st = 0; st < nst; ++st) {
                 const int last = st == nst - 1;
@@ -1141,7 +1141,7 @@ ens_status ens_mixture_host(int n, const double *lambdas, const uint64_t *counts
         s = ENS_ECUDA;
     if (s == ENS_OK) s = mixture_device(nullptr, n, d_lam, d_counts, d_mom, h, w, d_user, d_scr, out, st);
     cudaFreeAsync(mem, st);
-    cudaStreamSynchronize(st);
+    if (s != ENS_OK) cudaStreamSynchronize(st);   // (mixture_device synchronises when it succeeds)
     return s;
 }
 

@@ -73,7 +73,8 @@ const SizedOps *sized_ops(int N);   // nullptr for an unsupported size
 // z_mode: 0 persistent, 1 row groups, 2 persistent with the second warp plan).
 void launch_pass(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, int stage, int last, int arg,
                  cudaStream_t s);
-void launch_state_sums(const Geo &g, MemberDev *md, cudaStream_t s);
+// nblk: partial sums per member that launch_finish reads
+void launch_state_sums(const Geo &g, MemberDev *md, int nblk, cudaStream_t s);
 void launch_finish(MemberDev *md, int nmembers, const double *partial, int partial_blocks, int stage, int last,
                    int mode, cudaStream_t s);
 void launch_ic(const Geo &g, MemberDev *md, cudaStream_t s);

@@ -237,8 +237,9 @@ ens_status ens_step_host(ens_ctx *ctx, const void *host_in, void *host_out, size
  *                   instead of two; z_ctas_per_sm up to its own limit).
  * For N <= 64, z_variant 0 with tile_y 16 runs the inverse y, z and forward y
  * passes of a stage as one launch (a plane of constant x in shared memory;
- * z_ctas_per_sm unused but kept, and checked); every other combination, and
- * ens_run_pass, launches them one by one.
+ * z_ctas_per_sm unused but kept, and checked), and with fx_split 0, tile_x 16
+ * and plan_x 0 the last pass of a stage does the next stage's inverse x pass too;
+ * every other combination, and ens_run_pass, launches them one by one.
  * Every variant computes the same transforms; the FP64 energy sums of the
  * update pass are accumulated over tile_x-dependent CTA partials, so
  * changing tile_x changes their rounding order (fields agree to FP32
@@ -270,7 +271,7 @@ typedef struct {
 } ens_tuning;
 /* Current tuning.  At creation: tiles 16 (tile_x 8 for N >= 384), persistent z
  * pass at its occupancy limit (z_variant 2 where it exists, else 0), fx_split 1
- * for N >= 256 and for N = 64 with 8 members or more, parallel groups unless one of them has N >= 256. */
+ * for N >= 256 and for N = 64 with 12 members or more, parallel groups unless one of them has N >= 256. */
 ens_status ens_get_tuning(const ens_ctx *ctx, ens_tuning *out);
 /* Install a tuning (for instance one cached from an earlier ens_autotune on
  * the same device and member set).  ENS_EINVAL (not sticky, previous tuning

@@ -174,9 +174,11 @@ ens_status validate(const ens_member_desc *m, int n, const ens_hist_spec *h, std
 //                  against 1282 us per stage at 16 x 256^3, 235 / 304 at 384^3,
 //                  544 / 750 at 512^3); below that the transformed modes are a
 //                  larger part of the traffic than the waits (128^3: 242 / 212 us
-//                  at 24 members), but for 64^3 from 8 members on, where the fused
-//                  pass's small CTAs wait longest (step of 16 members 269 / 290
-//                  us, of 4 members 107 / 103)
+//                  at 24 members), and up to 64^3 the fused pass also starts the
+//                  next stage (k_chain), but for 64^3 from 12 members on, where its
+//                  CTAs wait on their state reads more than the saved launch and
+//                  read give (step of 16 members 267 split / 282 chained us, of 8
+//                  members 161 / 151, of one 77 / 58)
 //   z pass         the two-pass warp plan where there is one (256^3: 1418
 //                  against 1600 us per stage at 16 members, 96 / 109 at one)
 //   inverse x      8 columns at 384^3 and 512^3, where a 16-column tile leaves
@@ -186,7 +188,7 @@ void default_variants(Geo &g)
     g.tile_x = g.N >= 384 ? 8 : kTile;
     g.tile_y = kTile;
     g.plan_x = 0;
-    g.fx_split = g.N >= 256 || (g.N == 64 && g.members >= 8) ? 1 : 0;
+    g.fx_split = g.N >= 256 || (g.N == 64 && g.members >= 12) ? 1 : 0;
     g.z_mode = zplan_variant_available(g.N) ? 2 : 0;
 }
 // Grid sizes one after another as soon as one of them fills the GPU by itself
@@ -342,17 +344,26 @@ Geo single(const ens_ctx *ctx, int i)
     return g;
 }
 
+// One RK stage of a group, its end included.
 void record_group_stage(ens_ctx *ctx, const Geo &g, int st, int last, cudaStream_t s)
 {
-    launch_pass(Pass::IX, 0, g, ctx->md, nullptr, st, last, st > 0 ? 1 : 0, s);
+    const bool chain = chain_fused(g);
+    if (!chain || st == 0) launch_pass(Pass::IX, 0, g, ctx->md, nullptr, st, last, st > 0 ? 1 : 0, s);
     if (plane_fused(g)) {
-        launch_pass(Pass::PLANE, 0, g, ctx->md, nullptr, st, last, 0, s);
+        launch_pass(Pass::PLANE, 0, g, ctx->md, nullptr, st, last, chain && st > 0 ? 1 : 0, s);
     } else {
         launch_pass(Pass::IY, 0, g, ctx->md, nullptr, st, last, 6, s);
         launch_pass(Pass::Z, 0, g, ctx->md, nullptr, st, last, 0, s);
         launch_pass(Pass::FY, 0, g, ctx->md, nullptr, st, last, 0, s);
     }
+    if (chain && !last) {
+        // the stage's end comes with the next stage's PLANE launch
+        launch_pass(Pass::CHAIN, 0, g, ctx->md, nullptr, st, last, 0, s);
+        return;
+    }
     launch_pass(Pass::FX, 0, g, ctx->md, nullptr, st, last, 0, s);
+    launch_finish(ctx->md + g.first, g.members, ctx->partial + (size_t)g.first * ctx->partial_blocks * 4,
+                  ctx->partial_blocks, st, last, 0, s);
 }
 
 // One step with the persistent stage kernel: per RK stage, the work counters
@@ -378,9 +389,9 @@ void record_step_persistent(ens_ctx *ctx, cudaStream_t s)
 }
 
 // One step.  Groups of different grid size are independent until the
-// per-member stage reduction, so with several groups each group's pass chain
+// end of a stage, so with several groups each group's pass chain
 // runs on its own stream (a parallel branch of the captured graph), joined
-// before the reduction of every stage.
+// after every stage.
 void record_step(ens_ctx *ctx, cudaStream_t s)
 {
     if (ctx->persistent) {
@@ -388,7 +399,6 @@ void record_step(ens_ctx *ctx, cudaStream_t s)
         return;
     }
     const int nst = ctx->rk;
-    const int n = (int)ctx->desc.size();
     const int ng = (int)ctx->groups.size();
     for (int st = 0; st < nst; ++st) {
         const int last = st == nst - 1;
@@ -404,7 +414,6 @@ void record_step(ens_ctx *ctx, cudaStream_t s)
             record_group_stage(ctx, ctx->groups[0].geo, st, last, s);
             for (int gi = 1; gi < ng; ++gi) cudaStreamWaitEvent(s, ctx->ev_join[gi], 0);
         }
-        launch_finish(ctx->md, n, ctx->partial, ctx->partial_blocks, st, last, 0, s);
     }
 }
 
@@ -416,7 +425,6 @@ void record_step_sequential(ens_ctx *ctx, cudaStream_t s)
     for (int st = 0; st < nst; ++st) {
         const int last = st == nst - 1;
         for (int i = 0; i < n; ++i) record_group_stage(ctx, single(ctx, i), st, last, s);
-        launch_finish(ctx->md, n, ctx->partial, ctx->partial_blocks, st, last, 0, s);
     }
 }
 
@@ -707,9 +715,13 @@ int ens_kernels_per_step(const ens_ctx *ctx)
 {
     if (!ctx) return 0;
     if (ctx->persistent) return ctx->rk;   // one persistent launch per stage
-    int per_stage = 1;   // the per-member stage reduction
-    for (auto &gr : ctx->groups) per_stage += (plane_fused(gr.geo) ? 3 : 5) + (gr.geo.fx_split == 1 ? 1 : 0);
-    return ctx->rk * per_stage;
+    int total = 0;
+    for (auto &gr : ctx->groups) {
+        const Geo &g = gr.geo;
+        if (chain_fused(g)) total += 2 * ctx->rk + 2;   // IX, (PLANE, CHAIN) per stage, FX last, the end
+        else total += ctx->rk * ((plane_fused(g) ? 3 : 5) + (g.fx_split == 1 ? 1 : 0) + 1);
+    }
+    return total;
 }
 
 ens_status ens_step_sequential(ens_ctx *ctx, int nsteps)
@@ -856,7 +868,6 @@ ens_status ens_step_host(ens_ctx *ctx, const void *host_in, void *host_out, size
             for (int st = 0; st < nst; ++st) {
                 const int last = st == nst - 1;
                 record_group_stage(ctx, g, st, last, ctx->stream);
-                launch_finish(md, cnt, part, PB, st, last, 0, ctx->stream);
             }
             ENS_CUDA(ctx, cudaEventRecord(ctx->ev_done[ci], ctx->stream));
             ENS_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_out, ctx->ev_done[ci], 0));

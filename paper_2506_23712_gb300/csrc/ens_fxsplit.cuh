@@ -60,51 +60,6 @@ constexpr int update_blocks()
     return (int)((Dims<N>::SU + kUpdChunk - 1) / kUpdChunk);
 }
 
-// the update of one kept mode (Sec. IV): Leray projection of the nonlinear
-// term, band forcing, one integrating-factor RK stage; returns |u|^2 of the
-// result (both Hermitian halves counted by the caller)
-struct UpdCoef {
-    float inv_n3, dtf, alpha, nu, a, b, ha, hb;
-    int blo, bhi;
-};
-
-__device__ __forceinline__ float update_mode(const UpdCoef &c, int kx, int ky, int kz, float2 (&n)[3],
-                                             const float2 (&un)[3], const float2 (&us)[3], float2 (&out)[3],
-                                             bool &band, float &k2out)
-{
-    const float fk[3] = {(float)kx, (float)ky, (float)kz};
-    const int k2i = kx * kx + ky * ky + kz * kz;
-    const float k2 = (float)k2i;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) n[q] = cscale(n[q], c.inv_n3);
-    // Leray projection P_ij = delta_ij - k_i k_j / k^2; k = 0 held at zero
-    if (k2i == 0) {
-        n[0] = n[1] = n[2] = make_float2(0.f, 0.f);
-    } else {
-        const float inv = 1.f / k2;
-        const float dr = (fk[0] * n[0].x + fk[1] * n[1].x + fk[2] * n[2].x) * inv;
-        const float di = (fk[0] * n[0].y + fk[1] * n[1].y + fk[2] * n[2].y) * inv;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) n[q] = make_float2(n[q].x - fk[q] * dr, n[q].y - fk[q] * di);
-    }
-    band = k2i >= c.blo && k2i <= c.bhi;
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-        if (band) n[q] = make_float2(n[q].x + c.alpha * us[q].x, n[q].y + c.alpha * us[q].y);
-    const IfCoef ic = if_coef(StageCoef{c.a, c.ha, c.b, c.hb}, c.nu, k2, c.dtf);
-    float a2 = 0.f;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const float rx = us[q].x + c.dtf * n[q].x, ry = us[q].y + c.dtf * n[q].y;
-        const float ox = if_combine(ic, un[q].x, rx);
-        const float oy = if_combine(ic, un[q].y, ry);
-        out[q] = make_float2(ox, oy);
-        a2 += ox * ox + oy * oy;
-    }
-    k2out = k2;
-    return a2;
-}
-
 // grid (update_blocks<N>(), members), block kUpdThreads.  Thread t takes
 // the mode pairs (2j, 2j + 1), j = first + t + u * kUpdThreads: 16-byte
 // loads and stores, and every load of a pair issued before its arithmetic.
@@ -118,19 +73,7 @@ k_update(Geo g, MemberDev *md, int stage, int last_stage)
     static_assert(D::NZP % 2 == 0 && D::SU % 2 == 0, "mode pairs must not straddle a row");
     __shared__ double scratch[(kUpdThreads / 32) * 3];
     const int m = blockIdx.y;
-    const MemberDev &d = md[g.first + m];
-    const StageCoef co = stage_coef(d.rk, stage);
-    UpdCoef c;
-    c.inv_n3 = 1.0f / ((float)N * (float)N * (float)N);
-    c.dtf = (float)member_dt(d, N);
-    c.alpha = (float)d.alpha;
-    c.nu = (float)d.nu;
-    c.a = co.a;
-    c.b = co.b;
-    c.ha = co.ha;
-    c.hb = co.hb;
-    c.blo = d.band_lo2;
-    c.bhi = d.band_hi2;
+    const UpdCoef c = upd_coef<N>(md[g.first + m], stage);
     const float4 *nh = reinterpret_cast<const float4 *>(nhat_of<N>(g, m));
     const float4 *U = reinterpret_cast<const float4 *>(g.U + (long long)m * 3 * D::SU);
     const float4 *S = reinterpret_cast<const float4 *>(g.S + (long long)m * 3 * D::SU);

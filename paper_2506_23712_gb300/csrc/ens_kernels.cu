@@ -53,8 +53,7 @@ k_state_sums(Geo g, const MemberDev *md, int chunk)
     block_sum_to<3>(out, vals, scratch);
 }
 
-// End of a stage, a block per member: thread t adds the partials t, t +
-// blockDim, ..., then warps and warp sums in a fixed order.  One warp took 37 us
+// End of a stage, a block per member.  One warp took 37 us
 // per stage for the 7503 partials of a 512^3 member; 256 threads make its step
 // 8.79 ms from 9.00 (384^3: 4.01 from 4.10).  Where a member has few partials
 // (up to 64^3) one warp is the shorter chain (32^3: step 53 against 56 us).  (The
@@ -66,32 +65,7 @@ __global__ void __launch_bounds__(kFinishThreads)
 k_finish(MemberDev *md, const double *__restrict__ partial, int partial_blocks, int stage, int last_stage, int mode)
 {
     __shared__ double scratch[3 * kFinishThreads / 32];
-    MemberDev &d = md[blockIdx.x];
-    double v[3] = {0.0, 0.0, 0.0};
-    const double *pp = partial + (long long)blockIdx.x * partial_blocks * 4;
-    for (int k = threadIdx.x; k < d.nblk; k += blockDim.x) {
-        const double2 es = *reinterpret_cast<const double2 *>(pp + k * 4);
-        v[0] += es.x;
-        v[1] += es.y;
-        v[2] += pp[k * 4 + 2];
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) scratch[(threadIdx.x >> 5) * 3 + q] = v[q];
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    double e = 0.0, s = 0.0, b = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        e += scratch[w * 3];
-        s += scratch[w * 3 + 1];
-        b += scratch[w * 3 + 2];
-    }
-    finish_member(d, e, s, b, stage, last_stage, mode);
+    finish_block(md, partial, partial_blocks, stage, last_stage, mode, blockIdx.x, scratch);
 }
 
 // ---------------------------------------------------------------------------
@@ -376,6 +350,9 @@ bool plane_fused(const Geo &g)
 {
     return has_plane(g.N) && g.z_mode == 0 && g.tile_y == kTile && g.z_skip_member < 0;
 }
+
+// and its last pass does the next stage's inverse x transforms (k_chain)
+bool chain_fused(const Geo &g) { return plane_fused(g) && g.fx_split == 0 && g.tile_x == kTile && g.plan_x == 0; }
 
 int plan_threads(int N)
 {

@@ -705,6 +705,39 @@ __device__ __forceinline__ void finish_body(MemberDev *md, const double *partial
     if (lane == 0) finish_member(d, e, s, b, stage, last_stage, mode);
 }
 
+// The same by a whole block: thread t adds the partials t, t + blockDim, ...,
+// then warps and warp sums in a fixed order.  scratch: 3 blockDim / 32 doubles.
+__device__ __forceinline__ void finish_block(MemberDev *md, const double *__restrict__ partial, int partial_blocks,
+                                             int stage, int last_stage, int mode, int gm, double *scratch)
+{
+    MemberDev &d = md[gm];
+    double v[3] = {0.0, 0.0, 0.0};
+    const double *pp = partial + (long long)gm * partial_blocks * 4;
+    for (int k = threadIdx.x; k < d.nblk; k += blockDim.x) {
+        const double2 es = *reinterpret_cast<const double2 *>(pp + k * 4);
+        v[0] += es.x;
+        v[1] += es.y;
+        v[2] += pp[k * 4 + 2];
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) scratch[(threadIdx.x >> 5) * 3 + q] = v[q];
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double e = 0.0, s = 0.0, b = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        e += scratch[w * 3];
+        s += scratch[w * 3 + 1];
+        b += scratch[w * 3 + 2];
+    }
+    finish_member(d, e, s, b, stage, last_stage, mode);
+}
+
 template <int NW>
 __device__ __forceinline__ void block_sum_to(double *out, double (&vals)[NW], double *scratch)
 {
@@ -727,6 +760,69 @@ __device__ __forceinline__ void block_sum_to(double *out, double (&vals)[NW], do
         for (int w = 0; w < nw; ++w) s += scratch[w * NW + threadIdx.x];
         out[threadIdx.x] = s;
     }
+}
+
+// the update of one kept mode (Sec. IV): Leray projection of the nonlinear
+// term, band forcing, one integrating-factor RK stage; returns |u|^2 of the
+// result (both Hermitian halves counted by the caller)
+struct UpdCoef {
+    float inv_n3, dtf, alpha, nu, a, b, ha, hb;
+    int blo, bhi;
+};
+
+__device__ __forceinline__ float update_mode(const UpdCoef &c, int kx, int ky, int kz, float2 (&n)[3],
+                                             const float2 (&un)[3], const float2 (&us)[3], float2 (&out)[3],
+                                             bool &band, float &k2out)
+{
+    const float fk[3] = {(float)kx, (float)ky, (float)kz};
+    const int k2i = kx * kx + ky * ky + kz * kz;
+    const float k2 = (float)k2i;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) n[q] = cscale(n[q], c.inv_n3);
+    // Leray projection P_ij = delta_ij - k_i k_j / k^2; k = 0 held at zero
+    if (k2i == 0) {
+        n[0] = n[1] = n[2] = make_float2(0.f, 0.f);
+    } else {
+        const float inv = 1.f / k2;
+        const float dr = (fk[0] * n[0].x + fk[1] * n[1].x + fk[2] * n[2].x) * inv;
+        const float di = (fk[0] * n[0].y + fk[1] * n[1].y + fk[2] * n[2].y) * inv;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) n[q] = make_float2(n[q].x - fk[q] * dr, n[q].y - fk[q] * di);
+    }
+    band = k2i >= c.blo && k2i <= c.bhi;
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        if (band) n[q] = make_float2(n[q].x + c.alpha * us[q].x, n[q].y + c.alpha * us[q].y);
+    const IfCoef ic = if_coef(StageCoef{c.a, c.ha, c.b, c.hb}, c.nu, k2, c.dtf);
+    float a2 = 0.f;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float rx = us[q].x + c.dtf * n[q].x, ry = us[q].y + c.dtf * n[q].y;
+        const float ox = if_combine(ic, un[q].x, rx);
+        const float oy = if_combine(ic, un[q].y, ry);
+        out[q] = make_float2(ox, oy);
+        a2 += ox * ox + oy * oy;
+    }
+    k2out = k2;
+    return a2;
+}
+
+template <int N>
+__device__ __forceinline__ UpdCoef upd_coef(const MemberDev &d, int stage)
+{
+    const StageCoef co = stage_coef(d.rk, stage);
+    UpdCoef c;
+    c.inv_n3 = 1.0f / ((float)N * (float)N * (float)N);
+    c.dtf = (float)member_dt(d, N);
+    c.alpha = (float)d.alpha;
+    c.nu = (float)d.nu;
+    c.a = co.a;
+    c.b = co.b;
+    c.ha = co.ha;
+    c.hb = co.hb;
+    c.blo = d.band_lo2;
+    c.bhi = d.band_hi2;
+    return c;
 }
 
 template <int N, int MODE, int T, int VAR = 0>

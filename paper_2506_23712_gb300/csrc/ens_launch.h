@@ -5,7 +5,7 @@
 
 namespace ens {
 
-enum class Pass { IX, IY, Z, FY, FX, ZSTAT, PLANE };
+enum class Pass { IX, IY, Z, FY, FX, ZSTAT, PLANE, CHAIN };
 // IY mode of the statistics snapshot: the eight gradient components from the
 // six x-pass fields (u_i, i kx u_i)
 constexpr int kIYGrad = -1;
@@ -29,6 +29,7 @@ __host__ __device__ inline int mix_pdf_len(const MixPdfArgs &a) { return a.nq * 
 
 bool supported_n(int N);
 bool plane_fused(const Geo &g);   // the stage's middle runs as one PLANE launch
+bool chain_fused(const Geo &g);   // stages are linked by CHAIN launches
 int plan_threads(int N);
 int stats_blocks(int N);   // most partial-moment blocks per member
 size_t stats_smem(int N, int nq, int nt, int ng);   // shared memory per CTA of the statistics pass
@@ -67,7 +68,10 @@ const SizedOps *sized_ops(int N);   // nullptr for an unsupported size
 //   FY: forward along y of fields 0..2
 //   FX: mode 0 RK update, 1 right-hand side, 2 initial field, 3 plain transform
 //   ZSTAT: statistics
-//   PLANE: IY, Z mode 0 and FY in one launch (plane_fused(g) only)
+//   PLANE: IY, Z mode 0 and FY in one launch (plane_fused(g) only); arg 1: and the
+//          end of the stage before
+//   CHAIN: FX mode 0 of a stage that is not the last and IX of the next one
+//          (chain_fused(g) only)
 // The stage passes (IX mode 0, IY, FY, FX mode 0, Z mode 0) take their
 // variant from the group's tuning in g (tile_x, tile_y, plan_x, fx_split,
 // z_mode: 0 persistent, 1 row groups, 2 persistent with the second warp plan).

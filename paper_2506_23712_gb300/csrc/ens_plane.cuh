@@ -58,7 +58,9 @@ struct PlaneCfg {
     static_assert(CP::NP == 2 && WPadV<N, 0>::on && GR >= 1, "plans of the small sizes");
 };
 
-// grid (N, members), block 32 * WPB
+// grid (N + fin, members), block 32 * WPB.  fin: the block past the planes ends the
+// previous stage of its member (k_finish's work, which this pass does not need
+// and the next update does; a launch less)
 template <int N>
 __global__ void __launch_bounds__(32 * PlaneCfg<N>::WPB, 2)
 k_plane(Geo g, MemberDev *md, int stage_idx)
@@ -69,6 +71,11 @@ k_plane(Geo g, MemberDev *md, int stage_idx)
     using ZP = typename C::ZP;
     constexpr int V = CS::V, ZV = ZP::V, P = ZP::P, LPW = C::LPW, WPB = C::WPB, PITCH = C::PITCH, FS = C::FS;
     extern __shared__ __align__(16) float2 sm[];
+    if (blockIdx.x == N) {
+        finish_block(md, g.partial, g.partial_blocks, stage_idx - 1, 0, 0, g.first + blockIdx.y,
+                     reinterpret_cast<double *>(sm));
+        return;
+    }
     float2 *tw = sm, *plane = sm + N, *bufs = plane + 6 * FS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int x = blockIdx.x, m = blockIdx.y;
@@ -178,6 +185,181 @@ k_plane(Geo g, MemberDev *md, int stage_idx)
         store_kept<N, 0>(v, p, kz < D::NZS,
                          [&](auto s, float2 w) { at32(dst, off + (unsigned)CS::row(s.value) * row) = w; });
     }
+}
+
+// Last pass of a stage and first pass of the next in one launch, for the small
+// grids (N <= 64): forward x transform of the three components, RK update, and
+// the inverse x transforms of the next stage's u and omega, all on the same
+// columns, so the new state goes from the update into the transforms in
+// registers.  Thread (c, p) holds the positions p, p + P, p + 2 P, ... of its
+// column after the forward transform and needs the same ones before the
+// inverse (both passes of a two-pass plan deal positions out modulo P), and it
+// has all three components of each, which is what projection, forcing and
+// omega = i k x u need.  Registers bound the use: three lines of V values and
+// two in work (V = 8 up to 64^3).
+// One launch per stage less, the state's second read and the staged tile gone;
+// the stage's end moves into the next PLANE launch.  Step of 1 x 32^3 (RK2) 53.5
+// -> 43.1 us, 1 x 64^3 70.5 -> 57.6, 4 x 64^3 102.7 -> 88.2, 16 x 32^3 80 -> 66, 64 x 16^3 66
+// -> 58; from 12 members of 64^3 on the split last pass is faster.
+template <int N>
+struct ChainCfg {
+    static constexpr int T = kTile;
+    using CS = ColSlots<N, 0>;
+    static constexpr int V = CS::V, P = CS::P, TH = T * P;
+    // output slot that holds the position of input slot i
+    static __host__ __device__ constexpr int out_of(int i)
+    {
+        for (int o = 0; o < V; ++o)
+            if (CS::out(o) == CS::in(i)) return o;
+        return -1;
+    }
+    static constexpr size_t smem() { return smem_cols<N, T>(); }
+};
+
+// kept mode I of the three lines: the stage update of (n0, n1, n2) into u, and to dst
+template <int N, int I = 0>
+struct ChainUpdate {
+    using CS = ColSlots<N, 0>;
+    using D = Dims<N>;
+    static constexpr unsigned rowU = D::NK * D::NZP, SU = (unsigned)D::SU;
+    template <class Ld>
+    static __device__ __forceinline__ void run(const UpdCoef &c, int p, int ky, int kz, bool valid, bool stored,
+                                               unsigned off, const Ld &ld, float2 *dst, float2 *u0, float2 *u1,
+                                               float2 *u2, float &se, float &sd, float &sb)
+    {
+        if constexpr (I < CS::V) {
+            constexpr int C = CS::out(I);
+            constexpr auto kind = CS::kind(C);
+            if constexpr (kind == CS::kZero) {
+                u0[I] = u1[I] = u2[I] = make_float2(0.f, 0.f);
+            } else {
+                bool keep = true;
+                if constexpr (kind == CS::kLowMixed) keep = p <= CS::KC - C;
+                if constexpr (kind == CS::kNegMixed) keep = p >= N - CS::KC - C;
+                const unsigned o = off + (unsigned)CS::row(C) * rowU;
+                float2 un[3], us[3], n[3] = {u0[I], u1[I], u2[I]}, out[3];
+                ld(o, keep && valid, un, us);
+                bool band;
+                float k2;
+                const float a2 = update_mode(c, p + CS::wave(C), ky, kz, n, un, us, out, band, k2);
+                const bool real = keep && valid;
+                const float s = real ? (kz == 0 ? 1.f : 2.f) * a2 : 0.f;   // Hermitian multiplicity
+                se += 0.5f * s;
+                sd += c.nu * k2 * s;
+                if (band) sb += 0.5f * s;
+                u0[I] = real ? out[0] : make_float2(0.f, 0.f);
+                u1[I] = real ? out[1] : make_float2(0.f, 0.f);
+                u2[I] = real ? out[2] : make_float2(0.f, 0.f);
+                if (keep && stored) {
+                    at32(dst, o) = u0[I];
+                    at32(dst, o + SU) = u1[I];
+                    at32(dst, o + 2 * SU) = u2[I];
+                }
+            }
+            ChainUpdate<N, I + 1>::run(c, p, ky, kz, valid, stored, off, ld, dst, u0, u1, u2, se, sd, sb);
+        }
+    }
+};
+
+// first-pass inputs of an inverse transform from a line of modes u (output
+// slots): u, or (DX) i kx u
+template <int N, bool DX, int I = 0>
+__device__ __forceinline__ void chain_input(float2 *v, const float2 *u, int p)
+{
+    using CS = ColSlots<N, 0>;
+    if constexpr (I < CS::V) {
+        constexpr int C = CS::in(I), O = ChainCfg<N>::out_of(I);
+        if constexpr (CS::kind(C) == CS::kZero) v[I] = make_float2(0.f, 0.f);
+        else if constexpr (DX) v[I] = mul_i(cscale(u[O], (float)(p + CS::wave(C))));
+        else v[I] = u[O];
+        chain_input<N, DX, I + 1>(v, u, p);
+    }
+}
+
+// grid (NK NZp / 16, members), block 16 P
+template <int N>
+__global__ void __launch_bounds__(ChainCfg<N>::TH, 512 / ChainCfg<N>::TH)
+k_chain(Geo g, MemberDev *md, int stage)
+{
+    using C = ChainCfg<N>;
+    using CS = ColSlots<N, 0>;
+    using D = Dims<N>;
+    constexpr int V = C::V, T = C::T;
+    extern __shared__ __align__(16) float2 sm[];
+    float2 *tw = sm, *buf = sm + N;
+    load_col_twiddles<N, 0>(tw, g.tw);
+    const int c = threadIdx.x % T, p = threadIdx.x / T, m = blockIdx.y;
+    const unsigned col = blockIdx.x * T + c;                          // (ky, kz) flat
+    const int iy = col / D::NZP, kz = col % D::NZP;
+    const bool valid = kz < D::NZ, stored = kz < D::NZS;
+    float2 *A = g.A + (long long)m * kFields * D::SA;
+    const unsigned a0 = ((unsigned)iy * N + p) * D::NZP + kz;
+    auto at = [&](int pos) { return &buf[pos * T + c]; };
+    float2 u0[V], u1[V], u2[V];
+    auto load = [&](float2 *v, int q) {
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            v[i] = valid ? at32(A + q * D::SA, a0 + (unsigned)CS::in(i) * D::NZP) : make_float2(0.f, 0.f);
+    };
+    load(u0, 0);
+    load(u1, 1);
+    load(u2, 2);
+    fft_line<N, true, 0>(u0, p, tw, at);
+    fft_line<N, true, 0>(u1, p, tw, at);
+    fft_line<N, true, 0>(u2, p, tw, at);
+    // stage update: the new state to S (this is not the last stage) and in registers
+    const UpdCoef uc = upd_coef<N>(md[g.first + m], stage);
+    const int kyi = iy <= D::KC ? iy : iy - D::NK;
+    const long long base = (long long)m * 3 * D::SU;
+    const float2 *U = g.U + base, *S = g.S + base;
+    const unsigned SU = (unsigned)D::SU;
+    float se = 0.f, sd = 0.f, sb = 0.f;
+    auto ld = [&](unsigned o, bool ok, float2 (&un)[3], float2 (&us)[3]) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) un[q] = ok ? at32(U, o + q * SU) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) us[q] = ok && stage != 0 ? at32(S, o + q * SU) : un[q];
+    };
+    ChainUpdate<N>::run(uc, p, kyi, kz, valid, stored, p * (unsigned)(D::NK * D::NZP) + col, ld, g.S + base, u0, u1, u2,
+                        se, sd, sb);
+    // next stage: u and omega = i k x u, transformed along x (as inv_x_body)
+    const float ky = (float)kyi, kzf = (float)kz;
+    auto store = [&](const float2 *v, int f) {
+        if (stored) {
+            float2 *dst = A + f * D::SA;
+#pragma unroll
+            for (int i = 0; i < V; ++i) at32(dst, a0 + (unsigned)CS::out(i) * D::NZP) = v[i];
+        }
+    };
+    float2 Ua[V], Ub[V];
+    chain_input<N, false>(Ua, u1, p);
+    fft_line<N, false, 0, true>(Ua, p, tw, at);                       // uy
+    store(Ua, 1);
+    chain_input<N, false>(Ub, u2, p);
+    fft_line<N, false, 0, true>(Ub, p, tw, at);                       // uz
+    store(Ub, 2);
+#pragma unroll
+    for (int i = 0; i < V; ++i)
+        Ua[i] = mul_i(make_float2(ky * Ub[i].x - kzf * Ua[i].x, ky * Ub[i].y - kzf * Ua[i].y));
+    store(Ua, 3);                                                     // omega_x
+    chain_input<N, false>(Ua, u0, p);
+    fft_line<N, false, 0, true>(Ua, p, tw, at);                       // ux
+    store(Ua, 0);
+    chain_input<N, true>(Ub, u2, p);
+    fft_line<N, false, 0, true>(Ub, p, tw, at);                       // i kx uz
+#pragma unroll
+    for (int i = 0; i < V; ++i)
+        Ub[i] = make_float2(-kzf * Ua[i].y - Ub[i].x, kzf * Ua[i].x - Ub[i].y);
+    store(Ub, 4);                                                     // omega_y
+    chain_input<N, true>(Ub, u1, p);
+    fft_line<N, false, 0, true>(Ub, p, tw, at);                       // i kx uy
+#pragma unroll
+    for (int i = 0; i < V; ++i) Ub[i] = make_float2(Ub[i].x + ky * Ua[i].y, Ub[i].y - ky * Ua[i].x);
+    store(Ub, 5);                                                     // omega_z
+    __syncthreads();   // buf is reused as reduction scratch
+    double vals[3] = {(double)se, (double)sd, (double)sb};
+    double *out = g.partial + ((long long)(g.first + m) * g.partial_blocks + blockIdx.x) * 4;
+    block_sum_to<3>(out, vals, reinterpret_cast<double *>(buf));
 }
 
 }  // namespace ens

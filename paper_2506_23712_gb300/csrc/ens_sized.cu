@@ -52,8 +52,12 @@ cudaError_t prepare_variants()
 template <int M>
 cudaError_t prepare_plane()
 {
-    if constexpr (has_plane(M)) return allow_smem(k_plane<M>, PlaneCfg<M>::smem());
-    return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if constexpr (has_plane(M)) {
+        e = allow_smem(k_plane<M>, PlaneCfg<M>::smem());
+        if (e == cudaSuccess) e = allow_smem(k_chain<M>, ChainCfg<M>::smem());
+    }
+    return e;
 }
 
 cudaError_t prepare(int smem_optin)
@@ -87,9 +91,17 @@ cudaError_t prepare(int smem_optin)
 }
 
 template <int M>
-void launch_plane(const Geo &g, MemberDev *md, int stage, cudaStream_t s)
+void launch_plane(const Geo &g, MemberDev *md, int stage, int fin, cudaStream_t s)
 {
-    if constexpr (has_plane(M)) k_plane<M><<<dim3(M, g.members), 32 * PlaneCfg<M>::WPB, PlaneCfg<M>::smem(), s>>>(g, md, stage);
+    if constexpr (has_plane(M))
+        k_plane<M><<<dim3(M + fin, g.members), 32 * PlaneCfg<M>::WPB, PlaneCfg<M>::smem(), s>>>(g, md, stage);
+}
+
+template <int M>
+void launch_chain(const Geo &g, MemberDev *md, int stage, cudaStream_t s)
+{
+    if constexpr (has_plane(M))
+        k_chain<M><<<dim3(g.NK * g.NZp / ChainCfg<M>::T, g.members), ChainCfg<M>::TH, ChainCfg<M>::smem(), s>>>(g, md, stage);
 }
 
 template <int M>
@@ -220,7 +232,8 @@ void launch(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, 
         }
         break;
     }
-    case Pass::PLANE: launch_plane<N>(g, md, stage, s); break;
+    case Pass::PLANE: launch_plane<N>(g, md, stage, arg, s); break;
+    case Pass::CHAIN: launch_chain<N>(g, md, stage, s); break;
     case Pass::FX:
         switch (mode) {
         case 0:

@@ -202,7 +202,7 @@ __device__ __forceinline__ void inv_x_body(const Geo &g, int use_S, int bx, int 
                 return dx ? mul_i(cscale(u, (float)(p + CS::wave(s.value)))) : u;
             });
             fft_line<N, false, VAR, true>(v, p, tw, at);
-        } else {
+        } else if constexpr (N <= 256) {
             // statistics: every slot is multiplied and every butterfly formed, so
             // that the products by kx round as they always have (contracted into
             // the first additions) and the histogram counts stay the same
@@ -214,6 +214,18 @@ __device__ __forceinline__ void inv_x_body(const Geo &g, int use_S, int bx, int 
             } else {
                 fft_line<N, false, VAR, true>(v, p, tw, at);
             }
+        } else {
+            // (the three-pass plans contract them differently once the compiler
+            // knows which slots are zero: their rows are checked at run time)
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const int pos = PI::in_pos(p, i), kxi = pos <= N / 2 ? pos : pos - N;
+                const bool keep = kxi >= -Dims<N>::KC && kxi <= Dims<N>::KC;
+                const int ix = kxi >= 0 ? kxi : kxi + Dims<N>::NK;
+                const float2 u = keep ? tile[q * per + ix * T + c] : make_float2(0.f, 0.f);
+                v[i] = dx ? mul_i(cscale(u, (float)kxi)) : u;
+            }
+            fft_line<N, false, VAR, false>(v, p, tw, at);
         }
     };
     auto store = [&](const float2 *v, int f) {

@@ -304,8 +304,21 @@ __global__ void k_softmax_ce(const float *logit, const float *target, int nq, in
     const int len = kind == 0 ? nq * nq : nt;
     __shared__ float red[32];
     __shared__ float bval;
+    // up to kKeep logits per thread stay in registers between the three sweeps
+    constexpr int kKeep = 8;
+    const bool held = len <= kKeep * (int)blockDim.x;
+    float keep[kKeep];
     float mx = -INFINITY;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) mx = fmaxf(mx, logit[off + i]);
+    if (held) {
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = threadIdx.x + k * blockDim.x;
+            keep[k] = i < len ? logit[off + i] : -INFINITY;
+            mx = fmaxf(mx, keep[k]);
+        }
+    } else {
+        for (int i = threadIdx.x; i < len; i += blockDim.x) mx = fmaxf(mx, logit[off + i]);
+    }
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
     __syncthreads();
@@ -317,7 +330,13 @@ __global__ void k_softmax_ce(const float *logit, const float *target, int nq, in
     __syncthreads();
     mx = bval;
     float se = 0.f;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) se += __expf(logit[off + i] - mx);
+    if (held) {
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k)
+            if (threadIdx.x + k * blockDim.x < len) se += __expf(keep[k] - mx);
+    } else {
+        for (int i = threadIdx.x; i < len; i += blockDim.x) se += __expf(logit[off + i] - mx);
+    }
     for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = se;
@@ -330,15 +349,30 @@ __global__ void k_softmax_ce(const float *logit, const float *target, int nq, in
     __syncthreads();
     const float lse = mx + __logf(bval);
     float l = 0.f;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const float lq = logit[off + i] - lse;
+    const float w_hi = (float)weight, w_lo = (float)(weight - (double)w_hi);
+    auto out = [&](int i, float z) {
+        const float lq = z - lse;
         const float qi = __expf(lq);
         if (q) q[off + i] = qi;
         if (target) {
             const float p = target[off + i];
             if (p > 0.f) l -= p * lq;
-            if (dlogit) dlogit[off + i] = (float)((qi - p) * weight);
+            if (dlogit) {
+                // (qi - p) weight with the FP64 weight as two FP32 parts: FP64 runs on
+                // two lanes per SM and clock here
+                const float d = qi - p;
+                dlogit[off + i] = fmaf(d, w_hi, d * w_lo);
+            }
         }
+    };
+    if (held) {
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = threadIdx.x + k * blockDim.x;
+            if (i < len) out(i, keep[k]);
+        }
+    } else {
+        for (int i = threadIdx.x; i < len; i += blockDim.x) out(i, logit[off + i]);
     }
     if (loss_partial) {
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
@@ -994,7 +1028,7 @@ long long pad128(long long r) { return (r + 127) / 128 * 128; }
 bool alloc_rows(ens_surrogate *S, const RowSpec &rs, long long rows, int groups)
 {
     return S->logit.need(sizeof(float) * rows) && S->q.need(sizeof(float) * rows) &&
-           S->ftab.need(sizeof(uint4) * (kIn / 8) * rs.per_member) && S->loss.need(sizeof(double) * groups);
+           S->ftab.need(sizeof(uint4) * (kIn / 8) * rs.per_member) && S->loss.need(sizeof(double) * (groups + 1));
 }
 
 // CTAs per layer of the weight-gradient kernel: one wave over the SMs, in
@@ -1117,7 +1151,8 @@ void loss_grad_kernels(ens_surrogate *S, const RowSpec &rs, int n, long long row
                                                      S->dlogit.as<float>(), im, S->head_part.as<float>(), S->err);
     const WgradSplits sp = wgrad_splits(S, rows / 64);
     k_mlp_wgrad<<<sp.n[0] + sp.n[1] + sp.n[2], kWgThreads, kWgSmem, s>>>(im, rows / 64, sp, S->part.as<float>(), S->err);
-    k_grad_sum<<<blocks(S->L.total, 256), 256, 0, s>>>(S->part.as<float>(), sp, S->head_part.as<float>(), grid, S->g);
+    k_grad_sum<<<blocks(S->L.total, 256), 256, 0, s>>>(S->part.as<float>(), sp, S->head_part.as<float>(), grid, S->g,
+                                                       S->err, S->loss.as<double>() + 3 * n);
 }
 
 }  // namespace
@@ -1237,17 +1272,17 @@ ens_status ens_surrogate_loss_grad(ens_surrogate *S, int n, const double *lambda
     if (st != ENS_OK) return st;
     loss_grad_kernels(S, rs, n, rows, real, true);
     if (cudaGetLastError() != cudaSuccess) return ENS_ECUDA;
-    std::vector<double> lp(3 * n);
-    if (cudaMemcpyAsync(lp.data(), S->loss.p, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
+    std::vector<double> lp(3 * n + 1);   // group losses and the kernels' status
+    if (cudaMemcpyAsync(lp.data(), S->loss.p, sizeof(double) * lp.size(), cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
         return ENS_ECUDA;
     if (grad_host &&
         cudaMemcpyAsync(grad_host, S->g, sizeof(float) * S->L.total, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
         return ENS_ECUDA;
-    st = check_err(S);
-    if (st != ENS_OK) return st;
+    if (cudaStreamSynchronize(S->s) != cudaSuccess) return ENS_ECUDA;
+    if (lp[3 * n] != 0.0) return ENS_ETIMEOUT;
     if (loss) {
         double t = 0.0;
-        for (double v : lp) t += v;
+        for (int i = 0; i < 3 * n; ++i) t += lp[i];
         *loss = t;
     }
     return ENS_OK;

@@ -353,7 +353,7 @@ def measure_surrogate(E, ens, descs, torch, steps=800):
                                   "rows": rows_q, "flops_per_launch": infer_flops, "ms": infer_ms},
             "layer_gemm": {"kernel": "k_gemm_tc<256>", "shape": "%d x 256 x 256 BF16 -> FP32" % pad128(rows_q),
                            "ms": gemm_ms, "TFLOPs": gemm_tflops,
-                           "note": "training-path layer GEMM; FP32 output makes it HBM-bound (86 flop/B)"}}
+                           "note": "GEMM of the layer-by-layer check; FP32 output makes it HBM-bound (86 flop/B)"}}
 
 
 def held_out_gain(E, lams, counts, h, steps):

@@ -540,8 +540,8 @@ ens_status ens_surrogate_mixture(ens_surrogate *s, const ens_hist_spec *hist, co
  * hidden-layer GEMM of `rows` rows (rows x 256 x 256, BF16 in, FP32 out). */
 ens_status ens_surrogate_time_gemm(ens_surrogate *s, long long rows, int iters, double *ms);
 /* Logits [n][qr_bins^2 + 2 tail_bins] at n lambda values from the fused
- * inference kernel (fused != 0) or the layer-by-layer forward pass that
- * training uses (fused == 0); both round activations to BF16 the same way. */
+ * inference kernel (fused != 0) or a layer-by-layer forward pass that checks it
+ * (fused == 0); both round activations to BF16 the same way. */
 ens_status ens_surrogate_logits(ens_surrogate *s, int n, const double *lambdas, const ens_hist_spec *hist, int fused,
                                 float *logits);
 /* Average device time (ms) of one fused inference launch over nquad lambda

@@ -1067,15 +1067,19 @@ void pack_params(ens_surrogate *S)
     S->hbias_ok = false;
 }
 
+// buffers of the layer-by-layer forward pass
+bool alloc_layers(ens_surrogate *S, long long rows)
+{
+    return S->X.need(sizeof(__nv_bfloat16) * rows * kIn) && S->H.need(sizeof(__nv_bfloat16) * rows * kHid) &&
+           S->Z.need(sizeof(float) * rows * kHid) && S->Wb.need(sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid));
+}
+
 // layer-by-layer forward pass (one GEMM launch per layer) for `rows` padded
 // rows of the lambda values in S->lam: the check of the fused kernels
 bool forward_layers(ens_surrogate *S, const RowSpec &rs, int nlam, long long rows)
 {
     cudaStream_t s = S->s;
     const ParamLayout &L = S->L;
-    if (!S->X.need(sizeof(__nv_bfloat16) * rows * kIn) || !S->H.need(sizeof(__nv_bfloat16) * rows * kHid) ||
-        !S->Z.need(sizeof(float) * rows * kHid) || !S->Wb.need(sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid)))
-        return false;
     __nv_bfloat16 *X = S->X.as<__nv_bfloat16>(), *H = S->H.as<__nv_bfloat16>();
     __nv_bfloat16 *W1 = S->Wb.as<__nv_bfloat16>(), *W2 = W1 + kHid * kIn, *W3 = W2 + kHid * kHid;
     float *Z = S->Z.as<float>();
@@ -1379,9 +1383,7 @@ ens_status ens_surrogate_time_gemm(ens_surrogate *S, long long rows, int iters, 
 {
     if (!S || rows <= 0 || iters < 1 || !ms) return ENS_EINVAL;
     rows = pad128(rows);
-    if (!S->H.need(sizeof(__nv_bfloat16) * rows * kHid) || !S->Z.need(sizeof(float) * rows * kHid) ||
-        !S->Wb.need(sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid)))
-        return ENS_ENOMEM;
+    if (!alloc_layers(S, rows)) return ENS_ENOMEM;
     cudaMemsetAsync(S->H.p, 0, sizeof(__nv_bfloat16) * rows * kHid, S->s);
     cudaMemsetAsync(S->Wb.p, 0, sizeof(__nv_bfloat16) * (kHid * kIn + 2 * kHid * kHid), S->s);
     const __nv_bfloat16 *H = S->H.as<__nv_bfloat16>(), *W = S->Wb.as<__nv_bfloat16>() + kHid * kIn;
@@ -1413,6 +1415,7 @@ ens_status ens_surrogate_logits(ens_surrogate *S, int n, const double *lambdas, 
     if (!logits) return ENS_EINVAL;
     ens_status st = load_batch(S, n, lambdas, nullptr, h, &rows, &real, &rs);
     if (st != ENS_OK) return st;
+    if (!fused && !alloc_layers(S, rows)) return ENS_ENOMEM;
     if (fused ? !forward_fused(S, rs, real) : !forward_layers(S, rs, n, rows)) return ENS_ECUDA;
     if (cudaMemcpyAsync(logits, S->logit.p, sizeof(float) * real, cudaMemcpyDeviceToHost, S->s) != cudaSuccess)
         return ENS_ECUDA;

@@ -172,7 +172,7 @@ constexpr size_t smem_stats(int nq, int nt, int ng, int warps = SCfg<N>::WPB)
 // At most 8, and no more than the shared memory left beside the rest holds
 // (`room` bytes), down to one, which is the member's histogram layout itself.
 // 16 x 64^3 with 128 bins, whole snapshot: 1006 us with one copy, increments
-// aggregated by warp, and 32 CTAs; 431 us with 8 copies and 384 CTAs.
+// aggregated by warp, and 32 CTAs; 462 us with 8 copies and 384 CTAs.
 __host__ __device__ inline int grad_pitch(int ng) { return 2 * ng + 5; }
 inline int grad_copies(int ng, size_t room)
 {

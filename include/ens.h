@@ -264,7 +264,9 @@ typedef struct {
                           * pass counters); available when every grid size is
                           * 128, 256 or 384; the group variants below are then
                           * ignored (16-column tiles, 16 threads per FFT line,
-                          * the default z warp plan, the fused last pass) */
+                          * the default z warp plan, the fused last pass) by
+                          * ens_step and ens_step_nograph; ens_step_host and
+                          * ens_step_sequential launch pass by pass and follow them */
     ens_group_tuning group[ENS_MAX_GROUPS];   /* ascending N */
     double ms_per_step;  /* ens_autotune: mean step time of the winner, else 0 */
     int trials;          /* ens_autotune: configurations timed */

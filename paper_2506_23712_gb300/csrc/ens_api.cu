@@ -202,14 +202,6 @@ bool default_parallel(const std::vector<Group> &groups)
     return true;
 }
 
-// CTAs of a group's update pass that write partial sums
-int update_partials(const Geo &g, bool persistent)
-{
-    // the persistent stage kernel runs the fused update pass on 16-column tiles
-    if (persistent || g.fx_split == 2) return g.NK * g.NZp / 16;
-    return g.fx_split ? (int)((g.sU + kUpdChunk - 1) / kUpdChunk) : g.NK * g.NZp / g.tile_x;
-}
-
 // Group members by N (ascending), carve the workspace (base == nullptr: size only).
 size_t carve(const ens_member_desc *m, int n, const ens_hist_spec *h, char *base, ens_ctx *ctx)
 {
@@ -362,8 +354,7 @@ void record_group_stage(ens_ctx *ctx, const Geo &g, int st, int last, cudaStream
         return;
     }
     launch_pass(Pass::FX, 0, g, ctx->md, nullptr, st, last, 0, s);
-    launch_finish(ctx->md + g.first, g.members, ctx->partial + (size_t)g.first * ctx->partial_blocks * 4,
-                  ctx->partial_blocks, st, last, 0, s);
+    launch_stage_end(g, ctx->md, st, last, s);
 }
 
 // One step with the persistent stage kernel: per RK stage, the work counters
@@ -430,11 +421,7 @@ void record_step_sequential(ens_ctx *ctx, cudaStream_t s)
 
 ens_status resum(ens_ctx *ctx)
 {
-    // partial slots the sums kernel does not write must read as zero
-    ENS_CUDA(ctx, cudaMemsetAsync(ctx->partial, 0, sizeof(double) * ctx->desc.size() * ctx->partial_blocks * 4,
-                                  ctx->stream));
-    for (auto &gr : ctx->groups) launch_state_sums(gr.geo, ctx->md, update_partials(gr.geo, ctx->persistent), ctx->stream);
-    launch_finish(ctx->md, (int)ctx->desc.size(), ctx->partial, ctx->partial_blocks, 0, 0, 1, ctx->stream);
+    for (auto &gr : ctx->groups) launch_state_sums(gr.geo, ctx->md, ctx->stream);
     ENS_CUDA(ctx, cudaGetLastError());
     return ENS_OK;
 }
@@ -508,8 +495,6 @@ static ens_status init_context(ens_ctx *ctx, const ens_member_desc *m, int n, co
         x.index_in_group = ctx->member_local[i];
         x.seed = d.seed;
         x.init_energy = d.init_energy;
-        const Geo &g = ctx->groups[x.group].geo;
-        x.nblk = update_partials(g, false);   // update-pass CTAs (>= sums-kernel CTAs)
         x.dt = x.dt_fixed;
     }
     cudaStream_t st = ctx->stream;
@@ -843,7 +828,6 @@ ens_status ens_step_host(ens_ctx *ctx, const void *host_in, void *host_out, size
     // the uploads overwrite U: earlier work of the context stream first
     ENS_CUDA(ctx, cudaEventRecord(ctx->ev_start, ctx->stream));
     ENS_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_in, ctx->ev_start, 0));
-    const int PB = ctx->partial_blocks;
     const int nst = ctx->rk;
     const char *in = static_cast<const char *>(host_in);
     char *out = static_cast<char *>(host_out);
@@ -856,15 +840,11 @@ ens_status ens_step_host(ens_ctx *ctx, const void *host_in, void *host_out, size
         for (const int cnt : sched[gi]) {
             const Geo g = member_range(gr.geo, k0, cnt);
             const size_t b = per * cnt;
-            MemberDev *md = ctx->md + g.first;
-            double *part = ctx->partial + (size_t)g.first * PB * 4;
             ENS_CUDA(ctx, cudaMemcpyAsync(g.U, in + off, b, cudaMemcpyHostToDevice, ctx->copy_in));
             ENS_CUDA(ctx, cudaEventRecord(ctx->ev_in[ci], ctx->copy_in));
             ENS_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_in[ci], 0));
             // energy sums of the uploaded state, as after ens_set_state
-            ENS_CUDA(ctx, cudaMemsetAsync(part, 0, sizeof(double) * cnt * PB * 4, ctx->stream));
-            launch_state_sums(g, ctx->md, update_partials(g, ctx->persistent), ctx->stream);
-            launch_finish(md, cnt, part, PB, 0, 0, 1, ctx->stream);
+            launch_state_sums(g, ctx->md, ctx->stream);
             for (int st = 0; st < nst; ++st) {
                 const int last = st == nst - 1;
                 record_group_stage(ctx, g, st, last, ctx->stream);
@@ -1389,23 +1369,8 @@ ens_status tuning_valid(const ens_ctx *ctx, const ens_tuning *t, std::string &wh
     return ENS_OK;
 }
 
-// MemberDev::nblk of every member (one int per struct, strided) from its
-// group's current update-pass tile; synchronises
-ens_status sync_nblk(ens_ctx *ctx)
-{
-    for (auto &gr : ctx->groups) {
-        const Geo &g = gr.geo;
-        const int nblk = update_partials(g, ctx->persistent);
-        std::vector<int> v(g.members, nblk);
-        ENS_CUDA(ctx, cudaMemcpy2DAsync(&ctx->md[g.first].nblk, sizeof(MemberDev), v.data(), sizeof(int),
-                                        sizeof(int), g.members, cudaMemcpyHostToDevice, ctx->stream));
-    }
-    ENS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return ENS_OK;
-}
-
-// Install a (validated) tuning: pass variants per group, the update pass's
-// partial-sum count per member, and a fresh graph at the next ens_step.
+// Install a (validated) tuning: pass variants per group and a fresh graph at the
+// next ens_step; synchronises.
 ens_status apply_tuning(ens_ctx *ctx, const ens_tuning *t)
 {
     ctx->parallel_groups = t->parallel_groups;
@@ -1420,11 +1385,6 @@ ens_status apply_tuning(ens_ctx *ctx, const ens_tuning *t)
         g.z_mode = o.z_variant;
         g.z_ctas = o.z_ctas_per_sm * ctx->sms;
     }
-    const ens_status ns = sync_nblk(ctx);
-    if (ns != ENS_OK) return ns;
-    // slots a narrower tile wrote before must not leak into the reduction
-    ENS_CUDA(ctx, cudaMemsetAsync(ctx->partial, 0,
-                                  sizeof(double) * ctx->desc.size() * ctx->partial_blocks * 4, ctx->stream));
     ENS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (ctx->graph) {
         cudaGraphExecDestroy(ctx->graph);
@@ -1500,8 +1460,6 @@ ens_status ens_autotune(ens_ctx *ctx, int steps, ens_tuning *out)
     };
     // one trial: install, restore the snapshot, one untimed step, then the
     // mean of `steps` graph launches between two events
-    // (the snapshot holds the per-member partial-sum counts of the starting
-    // tuning, so the state is restored first and the tuning installed after)
     auto trial = [&](const ens_tuning &t) -> double {
         cudaError_t e = copy_state(false);
         if (e != cudaSuccess) return fail_cuda("autotune restore", e);
@@ -1798,8 +1756,7 @@ ens_status ens_load(ens_ctx *ctx, const char *path)
     hash = fnv1a(hash, counts.data(), sizeof(unsigned long long) * counts.size());
     hash = fnv1a(hash, mom.data(), sizeof(double) * mom.size());
     if (hash != h.payload_hash) return refuse("checksum mismatch");
-    // the member run state, spectral state and statistics as saved; the
-    // partial-sum counts follow this context's tuning
+    // the member run state, spectral state and statistics as saved
     const char *p = state.data();
     for (auto &gr : ctx->groups) {
         const size_t b = sizeof(float2) * 3 * gr.geo.sU * gr.geo.members;
@@ -1811,7 +1768,8 @@ ens_status ens_load(ens_ctx *ctx, const char *path)
                                   cudaMemcpyHostToDevice, ctx->stream));
     ENS_CUDA(ctx, cudaMemcpyAsync(ctx->moments, mom.data(), sizeof(double) * mom.size(), cudaMemcpyHostToDevice,
                                   ctx->stream));
-    return sync_nblk(ctx);
+    ENS_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return ENS_OK;
 }
 
 }  // extern "C"

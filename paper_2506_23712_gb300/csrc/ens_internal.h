@@ -20,7 +20,7 @@ struct MemberDev {
     int group, index_in_group;
     unsigned long long seed;     // initial-field seed
     double init_energy;
-    int nblk;                    // CTAs writing FP64 partial sums for this member
+    int reserved0;               // unused (checkpoints hold this struct: its layout stays)
     int band_lo2, band_hi2;      // forcing band as integer bounds on |k|^2
     int pad0;
     // run state

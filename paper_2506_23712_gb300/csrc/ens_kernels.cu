@@ -6,7 +6,6 @@
 #include "ens_stats.cuh"
 #include "ens_znl.cuh"
 
-#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -53,7 +52,8 @@ k_state_sums(Geo g, const MemberDev *md, int chunk)
     block_sum_to<3>(out, vals, scratch);
 }
 
-// End of a stage, a block per member.  One warp took 37 us
+// End of a stage, a block per member of a group, from the nblk partial sums per
+// member that the launch before wrote.  One warp took 37 us
 // per stage for the 7503 partials of a 512^3 member; 256 threads make its step
 // 8.79 ms from 9.00 (384^3: 4.01 from 4.10).  Where a member has few partials
 // (up to 64^3) one warp is the shorter chain (32^3: step 53 against 56 us).  (The
@@ -62,10 +62,11 @@ k_state_sums(Geo g, const MemberDev *md, int chunk)
 // a short kernel.)
 constexpr int kFinishThreads = 256;
 __global__ void __launch_bounds__(kFinishThreads)
-k_finish(MemberDev *md, const double *__restrict__ partial, int partial_blocks, int stage, int last_stage, int mode)
+k_finish(MemberDev *md, const double *__restrict__ partial, int partial_blocks, int nblk, int first, int stage,
+         int last_stage, int mode)
 {
     __shared__ double scratch[3 * kFinishThreads / 32];
-    finish_block(md, partial, partial_blocks, stage, last_stage, mode, blockIdx.x, scratch);
+    finish_block(md, partial, partial_blocks, nblk, stage, last_stage, mode, first + blockIdx.x, scratch);
 }
 
 // ---------------------------------------------------------------------------
@@ -414,18 +415,30 @@ void launch_pass(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev
     if (const SizedOps *o = sized_ops(g.N)) o->launch(pass, mode, g, md, h, stage, last, arg, s);
 }
 
-void launch_state_sums(const Geo &g, MemberDev *md, int nblk, cudaStream_t s)
+// Partial sums per member that FX mode 0 (or CHAIN) writes with g's variants:
+// one per column tile of the fused pass, one per kUpdChunk modes of the split one.
+static int update_partials(const Geo &g)
 {
-    // at most the partials that the end-of-stage sums read, and 2048 modes or more each
-    const int blocks = (int)std::min<long long>(nblk, (g.sU + kUpdChunk - 1) / kUpdChunk);
-    const int chunk = (int)((g.sU + blocks - 1) / blocks);
-    k_state_sums<<<dim3(blocks, g.members), kSumThreads, 0, s>>>(g, md, chunk);
+    if (g.fx_split == 1) return (int)((g.sU + kUpdChunk - 1) / kUpdChunk);
+    return g.NK * g.NZp / (g.fx_split == 2 ? kTile : g.tile_x);
 }
 
-void launch_finish(MemberDev *md, int nmembers, const double *partial, int partial_blocks, int stage, int last,
-                   int mode, cudaStream_t s)
+static void launch_finish(const Geo &g, MemberDev *md, int nblk, int stage, int last, int mode, cudaStream_t s)
 {
-    k_finish<<<nmembers, partial_blocks < 256 ? 32 : kFinishThreads, 0, s>>>(md, partial, partial_blocks, stage, last, mode);
+    k_finish<<<g.members, g.N <= 64 ? 32 : kFinishThreads, 0, s>>>(md, g.partial, g.partial_blocks, nblk, g.first, stage,
+                                                                   last, mode);
+}
+
+void launch_stage_end(const Geo &g, MemberDev *md, int stage, int last, cudaStream_t s)
+{
+    launch_finish(g, md, update_partials(g), stage, last, 0, s);
+}
+
+void launch_state_sums(const Geo &g, MemberDev *md, cudaStream_t s)
+{
+    const int blocks = (int)((g.sU + kUpdChunk - 1) / kUpdChunk);
+    k_state_sums<<<dim3(blocks, g.members), kSumThreads, 0, s>>>(g, md, (int)((g.sU + blocks - 1) / blocks));
+    launch_finish(g, md, blocks, 0, 0, 1, s);
 }
 
 void launch_ic(const Geo &g, MemberDev *md, cudaStream_t s)

@@ -693,17 +693,17 @@ __device__ __forceinline__ void finish_member(MemberDev &d, double e, double s, 
     }
 }
 
-// End of an RK stage for member gm (one warp, lane = 0..31): the FP64
-// partial sums of the update pass -> E, dissipation, band energy, the forcing
+// End of an RK stage for member gm (one warp, lane = 0..31): the nblk FP64
+// partial sums that the update pass wrote -> E, dissipation, band energy, the forcing
 // amplitude alpha = eps_inj / (2 E_B) of the next stage, the CFL step after the
 // first stage, time and step count after the last.
-__device__ __forceinline__ void finish_body(MemberDev *md, const double *partial, int partial_blocks, int stage,
-                                            int last_stage, int mode, int gm, int lane)
+__device__ __forceinline__ void finish_body(MemberDev *md, const double *partial, int partial_blocks, int nblk,
+                                            int stage, int last_stage, int mode, int gm, int lane)
 {
     MemberDev &d = md[gm];
     double e = 0.0, s = 0.0, b = 0.0;
     const double *pp = partial + (long long)gm * partial_blocks * 4;
-    for (int k = lane; k < d.nblk; k += 32) {
+    for (int k = lane; k < nblk; k += 32) {
         e += pp[k * 4 + 0];
         s += pp[k * 4 + 1];
         b += pp[k * 4 + 2];
@@ -720,12 +720,12 @@ __device__ __forceinline__ void finish_body(MemberDev *md, const double *partial
 // The same by a whole block: thread t adds the partials t, t + blockDim, ...,
 // then warps and warp sums in a fixed order.  scratch: 3 blockDim / 32 doubles.
 __device__ __forceinline__ void finish_block(MemberDev *md, const double *__restrict__ partial, int partial_blocks,
-                                             int stage, int last_stage, int mode, int gm, double *scratch)
+                                             int nblk, int stage, int last_stage, int mode, int gm, double *scratch)
 {
     MemberDev &d = md[gm];
     double v[3] = {0.0, 0.0, 0.0};
     const double *pp = partial + (long long)gm * partial_blocks * 4;
-    for (int k = threadIdx.x; k < d.nblk; k += blockDim.x) {
+    for (int k = threadIdx.x; k < nblk; k += blockDim.x) {
         const double2 es = *reinterpret_cast<const double2 *>(pp + k * 4);
         v[0] += es.x;
         v[1] += es.y;

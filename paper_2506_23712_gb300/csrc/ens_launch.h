@@ -77,10 +77,11 @@ const SizedOps *sized_ops(int N);   // nullptr for an unsupported size
 // z_mode: 0 persistent, 1 row groups, 2 persistent with the second warp plan).
 void launch_pass(Pass pass, int mode, const Geo &g, MemberDev *md, const HistDev *h, int stage, int last, int arg,
                  cudaStream_t s);
-// nblk: partial sums per member that launch_finish reads
-void launch_state_sums(const Geo &g, MemberDev *md, int nblk, cudaStream_t s);
-void launch_finish(MemberDev *md, int nmembers, const double *partial, int partial_blocks, int stage, int last,
-                   int mode, cudaStream_t s);
+// Run state of g's members from the partial sums of the update pass just launched
+// with the variants in g (the persistent stage kernel and PLANE do it themselves).
+void launch_stage_end(const Geo &g, MemberDev *md, int stage, int last, cudaStream_t s);
+// Energy sums of the state in U and the run state that follows from them.
+void launch_state_sums(const Geo &g, MemberDev *md, cudaStream_t s);
 void launch_ic(const Geo &g, MemberDev *md, cudaStream_t s);
 void launch_twiddles(float2 *tw, int N, cudaStream_t s);
 void launch_edges(float *eq, float *er, float *et, float *eg, int nq, int nt, int ng, double q_lim, double r_lim,

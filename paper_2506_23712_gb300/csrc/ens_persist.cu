@@ -102,8 +102,9 @@ __device__ __forceinline__ void run_item(int kind, const Geo &g, const PItem &it
         }
         break;
     default:
-        if (threadIdx.x < 32) finish_body(a.md, g.partial, g.partial_blocks, a.stage, a.last, 0, g.first + it.m,
-                                          threadIdx.x);
+        // one partial sum per 16-column tile of the kPFX items
+        if (threadIdx.x < 32) finish_body(a.md, g.partial, g.partial_blocks, g.NK * g.NZp / 16, a.stage, a.last, 0,
+                                          g.first + it.m, threadIdx.x);
         break;
     }
 }

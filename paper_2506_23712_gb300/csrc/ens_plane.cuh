@@ -72,7 +72,8 @@ k_plane(Geo g, MemberDev *md, int stage_idx)
     constexpr int V = CS::V, ZV = ZP::V, P = ZP::P, LPW = C::LPW, WPB = C::WPB, PITCH = C::PITCH, FS = C::FS;
     extern __shared__ __align__(16) float2 sm[];
     if (blockIdx.x == N) {
-        finish_block(md, g.partial, g.partial_blocks, stage_idx - 1, 0, 0, g.first + blockIdx.y,
+        // the partial sums of the k_chain launch before: one per column tile
+        finish_block(md, g.partial, g.partial_blocks, g.NK * g.NZp / kTile, stage_idx - 1, 0, 0, g.first + blockIdx.y,
                      reinterpret_cast<double *>(sm));
         return;
     }

@@ -289,9 +289,11 @@ k_mix_pdf(const unsigned long long *__restrict__ counts, const double *__restric
     const int L = a.counts_len;
     const int off_c = a.nq * a.nq + 2 * a.nt;
     __shared__ double wn[1024], part[TH], mom[kNMom];
+    __shared__ bool points[1024];
     for (int i = threadIdx.x; i < n; i += TH) {
         const double npts = (double)counts[(long long)i * L + off_c + 6];
         wn[i] = npts > 0.0 ? w[i] / npts : 0.0;
+        points[i] = npts > 0.0;
     }
     __syncthreads();
     if (blockIdx.x + 1 < gridDim.x) {
@@ -320,7 +322,11 @@ k_mix_pdf(const unsigned long long *__restrict__ counts, const double *__restric
     const int q = threadIdx.x % kNMom, slice = threadIdx.x / kNMom;
     double s = 0.0;
     if (slice < MS)
-        for (int i = slice; i < n; i += MS) s += wn[i] * moments[(long long)i * kNMom + q];
+        for (int i = slice; i < n; i += MS) {
+            const double mi = moments[(long long)i * kNMom + q];
+            // a member without points stays out, whatever its sums hold (0 x NaN is no zero)
+            if (points[i]) s += wn[i] * mi;
+        }
     part[threadIdx.x] = s;
     __syncthreads();
     if (slice == 0) {

@@ -321,7 +321,11 @@ ens_status ens_bin_check(ens_ctx *ctx, int axis, const float *values, int n, int
 ens_status ens_mixture(ens_ctx *ctx, const ens_weight_spec *w, ens_mixture_out *out);
 /* Mix statistics gathered elsewhere (e.g. from several processes): host
  * inputs lambdas [n], counts [n][counts_len], moments [n][ENS_NMOM]; runs on
- * the device with temporary device memory on `stream`.  n <= 1024. */
+ * the device with temporary device memory on `stream`.  n <= 1024.  That memory
+ * comes from a pool of the library's own, one per CUDA context: it keeps up to
+ * 32 MB of device memory between calls, until an ens_ctx of that CUDA context is
+ * destroyed (ens_destroy) or the context ends.  Synchronous; safe with several
+ * threads and streams, and after a device reset. */
 ens_status ens_mixture_host(int n, const double *lambdas, const uint64_t *counts, const double *moments,
                             const ens_hist_spec *hist, const ens_weight_spec *w, ens_mixture_out *out,
                             void *stream);

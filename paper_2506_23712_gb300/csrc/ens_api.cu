@@ -4,6 +4,8 @@
 #include "ens_launch.h"
 #include "ens_persist.h"
 
+#include <cudaTypedefs.h>
+
 #include <algorithm>
 #include <cstddef>
 #include <cmath>
@@ -583,6 +585,96 @@ static ens_status init_context(ens_ctx *ctx, const ens_member_desc *m, int n, co
     return ENS_OK;
 }
 
+// ---- device scratch of ens_mixture_host -------------------------------------
+// Memory pools of the library's own, which keep at most kScratchKeep bytes each
+// between calls (more goes back to the device at the next synchronisation), so
+// that repeated calls do not map and unmap their few megabytes each time (170 us
+// a call with the default pool, which keeps nothing; a pool maps 32 MB at a time,
+// and keeps nothing either where it may keep less than that).  Stream-ordered,
+// safe with several threads and streams.  One per CUDA context, found by the
+// context's id, which the driver never gives twice: a device reset ends the
+// context and its pool, and the next call then meets a new id (the context's
+// handle can stay the same).  What a pool keeps goes back when an ens_ctx is
+// destroyed.  Past kMaxScratchPools contexts, and where a pool cannot be made or
+// cannot grow, the default pool serves.
+
+namespace {
+
+constexpr int kMaxScratchPools = 64;
+constexpr unsigned long long kScratchKeep = 32ull << 20;
+struct ScratchPool {
+    unsigned long long ctx;
+    cudaMemPool_t pool;
+};
+std::mutex scratch_mu;
+ScratchPool scratch_pools[kMaxScratchPools];
+int scratch_count = 0;
+
+// id of the current CUDA context, 0 if there is none
+unsigned long long context_id()
+{
+    static const PFN_cuCtxGetId_v12000 get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<PFN_cuCtxGetId_v12000>(f);
+    }();
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// the current context's pool; without one: a new one, or nullptr (make: false)
+cudaMemPool_t scratch_pool(bool make)
+{
+    int dev = 0;
+    unsigned long long id = context_id();
+    if (!id && make) {   // before the first CUDA call, or after a reset: make the device's context current
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return nullptr;
+        id = context_id();
+    }
+    if (!id) return nullptr;
+    std::lock_guard<std::mutex> lock(scratch_mu);
+    for (int i = 0; i < scratch_count; ++i)
+        if (scratch_pools[i].ctx == id) return scratch_pools[i].pool;
+    if (!make || scratch_count == kMaxScratchPools) return nullptr;
+    cudaMemPoolProps pr{};
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = cudaGetDevice(&dev);
+    pr.location.id = dev;
+    if (e == cudaSuccess) e = cudaMemPoolCreate(&pool, &pr);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    unsigned long long keep = kScratchKeep;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    scratch_pools[scratch_count++] = ScratchPool{id, pool};
+    return pool;
+}
+
+cudaError_t scratch_alloc(void **mem, size_t bytes, cudaStream_t st)
+{
+    if (cudaMemPool_t pool = scratch_pool(true)) {
+        if (cudaMallocFromPoolAsync(mem, bytes, pool, st) == cudaSuccess) return cudaSuccess;
+        cudaGetLastError();
+    }
+    return cudaMallocAsync(mem, bytes, st);
+}
+
+// the memory that the current context's pool keeps, back to the device
+void scratch_trim()
+{
+    if (cudaMemPool_t pool = scratch_pool(false)) cudaMemPoolTrimTo(pool, 0);
+}
+
+}  // namespace
+
 extern "C" {
 
 const char *ens_status_string(ens_status s)
@@ -687,6 +779,7 @@ ens_status ens_destroy(ens_ctx *ctx)
     for (auto ev : ctx->ev_in) cudaEventDestroy(ev);
     for (auto ev : ctx->ev_done) cudaEventDestroy(ev);
     if (ctx->owns && ctx->workspace) cudaFree(ctx->workspace);
+    scratch_trim();
     delete ctx;
     return ENS_OK;
 }
@@ -1067,43 +1160,6 @@ ens_status ens_mixture(ens_ctx *ctx, const ens_weight_spec *w, ens_mixture_out *
     if (keep)
         for (int i = 0; i < n; ++i) keep[i] = wslot[slot_of(ctx, i)];
     return ENS_OK;
-}
-
-// Device scratch of ens_mixture_host: a memory pool of the library's own per
-// device, which keeps at most kScratchKeep bytes between calls (more goes back
-// to the device at the next synchronisation), so that repeated calls do not
-// map and unmap their few megabytes each time (170 us a call with the default
-// pool, which keeps nothing; a pool maps 32 MB at a time, and keeps nothing
-// either where it may keep less than that).  Stream-ordered, safe with several
-// threads and streams; the default pool where the device has no pools.
-static cudaError_t scratch_alloc(void **mem, size_t bytes, cudaStream_t st)
-{
-    constexpr int kMaxDev = 64;
-    constexpr unsigned long long kScratchKeep = 32ull << 20;
-    static std::mutex mu;
-    static cudaMemPool_t pools[kMaxDev] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    cudaMemPool_t pool = nullptr;
-    if (dev < kMaxDev) {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!pools[dev]) {
-            cudaMemPoolProps pr{};
-            pr.allocType = cudaMemAllocationTypePinned;
-            pr.location.type = cudaMemLocationTypeDevice;
-            pr.location.id = dev;
-            unsigned long long keep = kScratchKeep;
-            if (cudaMemPoolCreate(&pools[dev], &pr) != cudaSuccess) {
-                pools[dev] = nullptr;
-                cudaGetLastError();
-            } else {
-                cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
-            }
-        }
-        pool = pools[dev];
-    }
-    return pool ? cudaMallocFromPoolAsync(mem, bytes, pool, st) : cudaMallocAsync(mem, bytes, st);
 }
 
 ens_status ens_mixture_host(int n, const double *lambdas, const uint64_t *counts, const double *moments,

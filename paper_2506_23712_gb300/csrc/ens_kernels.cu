@@ -379,7 +379,7 @@ size_t stats_smem(int N, int nq, int nt, int ng)
 
 int stats_blocks(int N)
 {
-#define X(n) if (N == n) return stats_ctas<n>() * kStatsMaxSub;
+#define X(n) if (N == n) return stats_ctas<n>() * stats_most_sub<n>();
     ENS_SUPPORTED_N(X)
 #undef X
     return 0;

@@ -138,13 +138,16 @@ __host__ __device__ constexpr bool stats_split() { return N != 256; }
 // and flushing their histograms than the better balance gives.
 constexpr int kStatsMaxSub = 12;
 template <int N>
+constexpr int stats_most_sub()
+{
+    return !stats_split<N>() ? 1 : SCfg<N>::UNITS < kStatsMaxSub ? SCfg<N>::UNITS : kStatsMaxSub;
+}
+template <int N>
 int stats_sub(int members, int sms)
 {
-    if (!stats_split<N>()) return 1;
     const long long blocks = (long long)SCfg<N>::CTAS * members;
-    int sub = (int)((4LL * sms + blocks - 1) / blocks);
-    sub = sub < 1 ? 1 : sub > kStatsMaxSub ? kStatsMaxSub : sub;
-    return sub > SCfg<N>::UNITS ? SCfg<N>::UNITS : sub;
+    const int sub = (int)((4LL * sms + blocks - 1) / blocks);
+    return sub < 1 ? 1 : sub > stats_most_sub<N>() ? stats_most_sub<N>() : sub;
 }
 // warps of such a CTA
 template <int N>

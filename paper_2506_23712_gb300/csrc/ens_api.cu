@@ -179,8 +179,9 @@ ens_status validate(const ens_member_desc *m, int n, const ens_hist_spec *h, std
 //                  at 24 members), and up to 64^3 the fused pass also starts the
 //                  next stage (k_chain), but for 64^3 from 12 members on, where its
 //                  CTAs wait on their state reads more than the saved launch and
-//                  read give (step of 16 members 267 split / 282 chained us, of 8
-//                  members 161 / 151, of one 77 / 58)
+//                  read give (us per step of 16 members 260 split / 275 chained, of
+//                  12 members 216 / 211, of 8 members 154 / 148, of one 74 / 57:
+//                  the two cross between 12 and 16 members)
 //   z pass         the two-pass warp plan where there is one (256^3: 1418
 //                  against 1600 us per stage at 16 members, 96 / 109 at one)
 //   inverse x      8 columns at 384^3 and 512^3, where a 16-column tile leaves

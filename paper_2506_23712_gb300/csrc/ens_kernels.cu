@@ -53,10 +53,10 @@ k_state_sums(Geo g, const MemberDev *md, int chunk)
 }
 
 // End of a stage, a block per member of a group, from the nblk partial sums per
-// member that the launch before wrote.  One warp took 37 us
-// per stage for the 7503 partials of a 512^3 member; 256 threads make its step
-// 8.79 ms from 9.00 (384^3: 4.01 from 4.10).  Where a member has few partials
-// (up to 64^3) one warp is the shorter chain (32^3: step 53 against 56 us).  (The
+// member that the launch before wrote (9993 for a 512^3 member).  Steps with 256
+// threads against one warp: 512^3 8.80 / 9.25 ms, 384^3 4.00 / 4.17, 128^3 0.164 / 0.170.
+// Up to 64^3, with few partials, one warp is the shorter chain: 64 x 16^3 53.4 against
+// 54.7 us, 16 x 32^3 63.5 / 65.5, 16 x 64^3 260 / 263, 1 x 32^3 and one 64^3 the same.  (The
 // update pass's last CTA doing it, which saves the launch, measured 1% better at
 // 512^3 but 4% worse at 16 x 64^3: a fence, a counter and this sum at the end of
 // a short kernel.)

@@ -20,9 +20,11 @@
 // column, so the three phases need two block barriers between them and none
 // inside.  8 warps, two CTAs per SM.
 //
-// Measured (step, RK3 but for 32^3 x 1 with RK2): 16 x 64^3 346 -> 290 us (269 with
-// the split last pass), 4 x 64^3 125 -> 103, 64 x 64^3 1270 -> 1030, 1 x 32^3 64 -> 54,
-// 16 x 32^3 97 -> 80, 64 x 16^3 82 -> 66.
+// Measured (us per step, mean of 200 graph replays between two events, fixed step,
+// RK3 but for 1 x 32^3 with RK2; separate passes with 8-column y tiles -> this
+// kernel, both with the split last pass): 1 x 32^3 49 -> 41, 16 x 32^3 105 -> 85,
+// 64 x 16^3 101 -> 71, 1 x 64^3 84 -> 74, 4 x 64^3 123 -> 100, 16 x 64^3 338 -> 260,
+// 64 x 64^3 1208 -> 969.
 #pragma once
 
 #include "ens_znl.cuh"
@@ -199,9 +201,11 @@ k_plane(Geo g, MemberDev *md, int stage_idx)
 // omega = i k x u need.  Registers bound the use: three lines of V values and
 // two in work (V = 8 up to 64^3).
 // One launch per stage less, the state's second read and the staged tile gone;
-// the stage's end moves into the next PLANE launch.  Step of 1 x 32^3 (RK2) 53.5
-// -> 43.1 us, 1 x 64^3 70.5 -> 57.6, 4 x 64^3 102.7 -> 88.2, 16 x 32^3 80 -> 66, 64 x 16^3 66
-// -> 58; from 12 members of 64^3 on the split last pass is faster.
+// the stage's end moves into the next PLANE launch.  Step (measured as for k_plane;
+// fused last pass on 8-column tiles -> chained): 1 x 32^3 37 -> 31 us, 16 x 32^3 78 -> 64,
+// 64 x 16^3 63 -> 53, 1 x 64^3 74 -> 57, 4 x 64^3 102 -> 84.  With more members of 64^3
+// the split last pass catches up: chained against split 148 / 154 us at 8, 211 / 216
+// at 12, 275 / 260 at 16, 985 / 969 at 64.
 template <int N>
 struct ChainCfg {
     static constexpr int T = kTile;

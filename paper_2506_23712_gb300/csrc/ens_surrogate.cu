@@ -304,7 +304,9 @@ __global__ void k_softmax_ce(const float *logit, const float *target, int nq, in
     const int len = kind == 0 ? nq * nq : nt;
     __shared__ float red[32];
     __shared__ float bval;
-    // up to kKeep logits per thread stay in registers between the three sweeps
+    // up to kKeep logits per thread stay in registers between the three sweeps: every
+    // group of up to 8192 bins in training (1024 threads), of up to 2048 in inference
+    // (256 threads), where a longer group is read three times
     constexpr int kKeep = 8;
     const bool held = len <= kKeep * (int)blockDim.x;
     float keep[kKeep];

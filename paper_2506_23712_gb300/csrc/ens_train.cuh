@@ -95,8 +95,9 @@ struct TrainImages {
 // M2, M6) and never leave the tensor memory.  An epilogue loads its whole
 // accumulator A before its first chunk arrival, so the next product may start
 // on chunk 0 while the later chunks are still being formed; B is rewritten
-// only after every warp has read it (`feat` arrivals for M6, `fin` arrivals
-// for the next tile's M2).  Weight K-blocks stream through the three slots in
+// only after every warp has read it (`feat` arrivals for M6).  The next tile's
+// products, M3 included, wait for the `fin` arrivals behind E5; only its copies
+// run beside E5.  Weight K-blocks stream through the three slots in
 // the order of use, 17 per tile; M4 and M5 take 64 rows of the weight image
 // (four 8 KB pieces) as MN-major operands.  Every wait is bounded; a role
 // whose wait gives up sets *err and the CTA drains.
